@@ -19,12 +19,26 @@
 //
 // Pipelines: raw FP32 operand tiles arrive several stages ahead, by TMA
 // tensor copies that one producer thread issues (or, without TMA, by the
-// producers' own cp.async); four producer warps split them into the TF32
-// operand planes of a shared-memory stage and signal an mbarrier; one warp
-// issues the MMAs and
+// producers' own cp.async); groups of four producer warps split them into
+// the TF32 operand planes of a shared-memory stage and signal an mbarrier;
+// one warp issues the MMAs and
 // releases the stage with tcgen05.commit; two TMEM accumulators alternate so
 // that four more warps read one out while the MMAs fill the other.  Every
 // wait is bounded (tc.cuh).
+//
+// What bounds a k-step (8 complex values of K, 128 x 128 complex outputs):
+// the six MMAs take 770 cycles at the TF32 rate, the operand traffic through
+// shared memory about 1,000.  Measured on one GB300 (256^2 pixels, 128 elements
+// x 6 frequencies): contraction 375 -> 205 us a launch (137 -> 251 TFLOP/s),
+// J^H 354 -> 254 us, 1,200-1,400 cycles a k-step, from three changes: MMAs
+// issued by an elected lane of a converged warp from precomputed descriptor
+// words (see KStep); three producer groups, each converting every third k-step,
+// so that their chains of waits, loads, splits, stores and proxy fences run
+// side by side (one group: 2,200 cycles a k-step); and B blocks cut to the
+// elements there are (64 elements: half the MMA and operand work; the data
+// projection of 384^2 x 64 elements x 15 frequencies 1.60 -> 0.93 ms).  Eight
+// producer warps a group instead of four, and A kept in the collector buffer
+// between MMAs, changed nothing.
 #include <cstring>
 #include <mutex>
 #include <string>
@@ -45,34 +59,57 @@ constexpr int KS = 8;                 // complex values per k-step (TF32 K = 8)
 constexpr int PLANE = ROWS * 32;      // one 128-row operand block of a k-step
 constexpr int BROWS = 3 * ROWS;       // B stack [-Bi | Br | Bi]
 constexpr int BPLANE = BROWS * 32;
-constexpr uint32_t LBO_A = 16 * ROWS, LBO_B = 16 * BROWS, SBO = 128;
-constexpr uint32_t IDESC = tc::idesc_tf32(128, 256, false);
-// 4 producer warps, 1 MMA warp, 4 accumulator warps (drain / epilogue)
-constexpr int C_THREADS = 288;
-constexpr int C_TILE_STRIDE = 17;     // drain transpose tile: [32 rows][16 + 1] float2
+constexpr uint32_t LBO_A = 16 * ROWS, SBO = 128;
+// 3 groups of 4 producer warps (group p converts the k-steps g = p mod 3), 1
+// MMA warp, 4 accumulator warps (drain / epilogue)
+constexpr int GROUPS = 3;
+constexpr int MMA_WARP = 4 * GROUPS;
+constexpr int C_THREADS = 32 * (MMA_WARP + 5);
+constexpr int C_TILE_STRIDE = 9;      // drain transpose tile: [32 rows][8 + 1] float2
 constexpr int C_TILE_BYTES = 32 * C_TILE_STRIDE * 8;
 
+// B blocks hold a multiple of 8 rows (MMA N = twice that), so that few rows are
+// padding: 64 elements run at N = 128, 192 at two contraction tiles of N = 192.
+__host__ __device__ constexpr int round8(int n) { return (n + 7) & ~7; }
+
 // Operand planes inside a conversion stage: A = {Ar hi, Ar lo, Ai hi, Ai lo}
-// (one 128-row block each), then B hi and B lo (384 rows each).
-__device__ __forceinline__ void issue_kstep(uint32_t tmem, uint32_t a_base, uint32_t b_base,
-                                           uint32_t first) {
-  using namespace tc;
-  const uint64_t ar_h = sdesc(a_base + 0 * PLANE, LBO_A, SBO);
-  const uint64_t ar_l = sdesc(a_base + 1 * PLANE, LBO_A, SBO);
-  const uint64_t ai_h = sdesc(a_base + 2 * PLANE, LBO_A, SBO);
-  const uint64_t ai_l = sdesc(a_base + 3 * PLANE, LBO_A, SBO);
-  // [Br; Bi] starts at row 128 of the stack, [-Bi; Br] at row 0
-  const uint64_t b1_h = sdesc(b_base + 16 * ROWS, LBO_B, SBO);
-  const uint64_t b1_l = sdesc(b_base + BPLANE + 16 * ROWS, LBO_B, SBO);
-  const uint64_t b2_h = sdesc(b_base, LBO_B, SBO);
-  const uint64_t b2_l = sdesc(b_base + BPLANE, LBO_B, SBO);
-  mma_tf32(tmem, ar_h, b1_h, IDESC, first ? 0u : 1u);
-  mma_tf32(tmem, ar_h, b1_l, IDESC, 1u);
-  mma_tf32(tmem, ar_l, b1_h, IDESC, 1u);
-  mma_tf32(tmem, ai_h, b2_h, IDESC, 1u);
-  mma_tf32(tmem, ai_h, b2_l, IDESC, 1u);
-  mma_tf32(tmem, ai_l, b2_h, IDESC, 1u);
-}
+// (one 128-row block each), then B hi and B lo (3 nbr rows each: two
+// half-k-step planes of 48 nbr bytes, bplane(nbr) together).
+__device__ __forceinline__ uint32_t bplane(uint32_t nbr) { return 96 * nbr; }
+// nbr: rows of a B block; the accumulator is [nbr Re | nbr Im].  The MMAs are
+// issued by one elected lane of a warp that stays converged, from descriptors
+// whose high words are constant and whose low words differ by additions: with
+// a divergent lane 0 computing eight whole descriptors the issue took 1,350
+// cycles a k-step, more than the MMAs themselves.
+struct KStep {
+  uint32_t nbr, idesc, hi, lo_a, lo_b;  // lo_a, lo_b: address field still 0
+  __device__ __forceinline__ explicit KStep(uint32_t rows)
+      : nbr(rows), idesc(tc::idesc_tf32(ROWS, 2 * (int)rows, false)),
+        hi((uint32_t)(tc::sdesc(0, 0, SBO) >> 32)), lo_a((LBO_A >> 4) << 16),
+        lo_b((48 * rows >> 4) << 16) {}
+  __device__ __forceinline__ uint64_t desc(uint32_t lo) const {
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
+    return d;
+  }
+  __device__ __forceinline__ void issue(uint32_t tmem, uint32_t a_base, uint32_t b_base,
+                                        bool first) const {
+    using namespace tc;
+    // A planes one block apart; [Br; Bi] starts at row nbr of the stack,
+    // [-Bi; Br] at row 0, the lo parts bplane(nbr) bytes further
+    const uint32_t a = lo_a + (a_base >> 4), b = lo_b + (b_base >> 4);
+    const uint32_t bl = b + (bplane(nbr) >> 4);
+    const uint64_t ar_h = desc(a), ar_l = desc(a + (PLANE >> 4));
+    const uint64_t ai_h = desc(a + 2 * (PLANE >> 4)), ai_l = desc(a + 3 * (PLANE >> 4));
+    const uint64_t b1_h = desc(b + nbr), b1_l = desc(bl + nbr), b2_h = desc(b), b2_l = desc(bl);
+    mma_tf32(tmem, ar_h, b1_h, idesc, first ? 0u : 1u);
+    mma_tf32(tmem, ar_h, b1_l, idesc, 1u);
+    mma_tf32(tmem, ar_l, b1_h, idesc, 1u);
+    mma_tf32(tmem, ai_h, b2_h, idesc, 1u);
+    mma_tf32(tmem, ai_h, b2_l, idesc, 1u);
+    mma_tf32(tmem, ai_l, b2_h, idesc, 1u);
+  }
+};
 
 // Store 4 consecutive-k values of operand row `row` (hi and lo planes).
 __device__ __forceinline__ void put_a(uint32_t plane_hi, uint32_t plane_lo, int half, int row,
@@ -85,8 +122,8 @@ __device__ __forceinline__ void put_a(uint32_t plane_hi, uint32_t plane_lo, int 
   tc::sts128(plane_lo + off, l[0], l[1], l[2], l[3]);
 }
 
-// B row `row`: re and im parts into the [-Bi | Br | Bi] stack.
-__device__ __forceinline__ void put_b(uint32_t bhi, uint32_t blo, int half, int row,
+// B row `row` (of nbr): re and im parts into the [-Bi | Br | Bi] stack.
+__device__ __forceinline__ void put_b(uint32_t bhi, uint32_t blo, int half, int row, int nbr,
                                       const float (&re)[4], const float (&im)[4]) {
   float rh[4], rl[4], ih[4], il[4];
 #pragma unroll
@@ -94,13 +131,14 @@ __device__ __forceinline__ void put_b(uint32_t bhi, uint32_t blo, int half, int 
     tc::split_tf32(re[i], rh[i], rl[i]);
     tc::split_tf32(im[i], ih[i], il[i]);
   }
-  const uint32_t o = (uint32_t)(half * 16 * BROWS + 16 * row);
+  const uint32_t o = (uint32_t)(half * 48 * nbr + 16 * row);
+  const uint32_t o1 = o + 16 * (uint32_t)nbr, o2 = o + 32 * (uint32_t)nbr;
   tc::sts128(bhi + o, -ih[0], -ih[1], -ih[2], -ih[3]);
-  tc::sts128(bhi + o + 16 * ROWS, rh[0], rh[1], rh[2], rh[3]);
-  tc::sts128(bhi + o + 32 * ROWS, ih[0], ih[1], ih[2], ih[3]);
+  tc::sts128(bhi + o1, rh[0], rh[1], rh[2], rh[3]);
+  tc::sts128(bhi + o2, ih[0], ih[1], ih[2], ih[3]);
   tc::sts128(blo + o, -il[0], -il[1], -il[2], -il[3]);
-  tc::sts128(blo + o + 16 * ROWS, rl[0], rl[1], rl[2], rl[3]);
-  tc::sts128(blo + o + 32 * ROWS, il[0], il[1], il[2], il[3]);
+  tc::sts128(blo + o1, rl[0], rl[1], rl[2], rl[3]);
+  tc::sts128(blo + o2, il[0], il[1], il[2], il[3]);
 }
 
 __device__ __forceinline__ float4 lds128(uint32_t addr) {
@@ -121,21 +159,22 @@ __device__ __forceinline__ float2 lds64(uint32_t addr) {
 
 // ---------------------------------------------------------------------------
 // Contraction: one CTA per (pixel chunk s, tile pair (eb, jb), frequency l);
-// accumulator D[e][j] (128 x [128 Re | 128 Im]) over its pixel chunk,
-// written as FP32 partials part[s][l][e][j].
-// Raw stages: 128 rows of X (and of Q unless the two share rows) plus the
-// 8 weights a[n]; SHARED (X == Q, one element tile) keeps 8 stages in
-// flight, the general case 4; after them come the four drain warps'
-// transpose tiles.
+// accumulator D[e][j] (128 x [nbr Re | nbr Im]) over its pixel chunk,
+// written as FP32 partials part[s][l][e][j].  The n_elem rows are dealt
+// evenly over the tiles (tr rows each).
+// Raw stages (RN per producer group): 128 rows of X (and of Q unless the two
+// share rows), then the 8 weights a[n] of every stage, then the four drain
+// warps' transpose tiles.
 constexpr int C_CONV = 3;
 constexpr int C_RAWROW = 80;  // 8 complex (64 bytes) + 16 bytes of padding
 constexpr int C_CONV_BYTES = 4 * PLANE + 2 * BPLANE;
 template <bool SHARED> struct CRaw {
-  static constexpr int N = SHARED ? 8 : 4;
+  static constexpr int RN = SHARED ? 2 : 1;
+  static constexpr int N = GROUPS * RN;
   static constexpr int X = 0, Q = ROWS * C_RAWROW;
-  static constexpr int A = (SHARED ? 1 : 2) * ROWS * C_RAWROW;
-  static constexpr int BYTES = A + 64;
-  static constexpr int TILES = C_CONV * C_CONV_BYTES + N * BYTES;
+  static constexpr int BYTES = (SHARED ? 1 : 2) * ROWS * C_RAWROW;
+  static constexpr int AW = C_CONV * C_CONV_BYTES + N * BYTES;
+  static constexpr int TILES = AW + N * 64;
   static constexpr int SMEM = TILES + 4 * C_TILE_BYTES;
 };
 // Raw stages filled by TMA: rows of 64 bytes without padding, written with
@@ -143,15 +182,19 @@ template <bool SHARED> struct CRaw {
 // mod 4)), which keeps the producers' 16-byte row reads free of bank
 // conflicts; stages 1024-byte aligned for the swizzle pattern.
 template <bool SHARED> struct CRawT {
-  static constexpr int N = SHARED ? 8 : 4;
+  static constexpr int RN = SHARED ? 3 : 2;
+  static constexpr int N = GROUPS * RN;
   static constexpr int TILE = ROWS * 64;  // one operand's box
   static constexpr int X = 0, Q = TILE;
-  static constexpr int A = (SHARED ? 1 : 2) * TILE;
-  static constexpr int BYTES = ((A + 64 + 1023) / 1024) * 1024;
-  static constexpr int TX = (SHARED ? 1 : 2) * TILE;  // bytes the TMA copies deliver
-  static constexpr int TILES = C_CONV * C_CONV_BYTES + N * BYTES;
+  static constexpr int BYTES = (SHARED ? 1 : 2) * TILE;
+  static constexpr int TX = BYTES;  // bytes the TMA copies deliver
+  static constexpr int AW = C_CONV * C_CONV_BYTES + N * BYTES;
+  static constexpr int TILES = AW + N * 64;
   static constexpr int SMEM = TILES + 4 * C_TILE_BYTES;
 };
+static_assert(CRaw<true>::SMEM <= 226 * 1024 && CRaw<false>::SMEM <= 226 * 1024 &&
+              CRawT<true>::SMEM <= 226 * 1024 && CRawT<false>::SMEM <= 226 * 1024,
+              "dynamic shared memory beside the static barriers");
 // Byte offset of 16-byte chunk q of row r in a swizzled 64-byte-row tile.
 __device__ __forceinline__ uint32_t swz64(int r, int q) {
   return (uint32_t)(r * 64 + ((q ^ ((r >> 1) & 3)) << 4));
@@ -165,6 +208,7 @@ struct ContractArgs {
   int* err;
   long long N, chunk;
   int NE, n_freq;
+  int tr;           // rows per operand tile
   int sub_ks;       // k-steps per accumulation sub-chunk
   int stall;        // test of the failure path: withhold the first stage
 };
@@ -173,8 +217,8 @@ struct ContractArgs {
 // sub-chunks: while the MMA warp accumulates sub-chunk s into buffer s % 2,
 // four drain warps add buffer (s - 1) % 2 into the CTA's FP32 partial.  A
 // drain warp owns the 32 TMEM lanes of its quadrant (32 rows e) and moves
-// 16 columns at a time through a shared transpose tile, so that its global
-// read-modify-write covers two 128-byte row segments per instruction.
+// 8 columns at a time through a shared transpose tile, so that its global
+// read-modify-write covers four 64-byte row segments per instruction.
 // XTMA: the raw X (and Q) tiles arrive by TMA tensor copies (64-byte
 // swizzle) issued by one producer thread and completing on bar_raw; the
 // weights a still come by cp.async.  Otherwise every producer copies its
@@ -185,17 +229,21 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_contract_kernel(
     const __grid_constant__ CUtensorMap qmap) {
   using namespace tc;
   using RW = typename std::conditional<XTMA, CRawT<SHARED>, CRaw<SHARED>>::type;
-  constexpr int C_RAW = RW::N, C_RAW_BYTES = RW::BYTES;
-  constexpr int C_RAW_X = RW::X, C_RAW_Q = RW::Q, C_RAW_A = RW::A;
+  constexpr int RN = RW::RN, C_RAW_BYTES = RW::BYTES;
+  constexpr int C_RAW_X = RW::X, C_RAW_Q = RW::Q;
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t bar_full[C_CONV], bar_empty[C_CONV], bar_done[2],
-      bar_freed[2], bar_final, bar_raw[C_RAW];
+      bar_freed[2], bar_final, bar_raw[RW::N];
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int s = blockIdx.x, l = blockIdx.z;
   const int nbe = (p.NE + ROWS - 1) / ROWS;
   const int eb = blockIdx.y % nbe, jb = blockIdx.y / nbe;
+  const int er0 = eb * p.tr, jr0 = jb * p.tr;              // first rows of the tiles
+  const int ne = (p.NE - er0 < p.tr) ? p.NE - er0 : p.tr;  // rows of the e tile
+  const int nj = (p.NE - jr0 < p.tr) ? p.NE - jr0 : p.tr;
+  const int nbr = round8(nj);                              // rows of a B block
   const long long n_begin = (long long)s * p.chunk;
   const long long n_end = (n_begin + p.chunk < p.N) ? n_begin + p.chunk : p.N;
   const int nch = (n_begin < p.N) ? (int)((n_end - n_begin + KS - 1) / KS) : 0;
@@ -215,7 +263,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_contract_kernel(
     }
     mbar_init(smem_addr(&bar_final), 1);
     if (XTMA)
-      for (int i = 0; i < C_RAW; ++i) mbar_init(smem_addr(&bar_raw[i]), 1);
+      for (int i = 0; i < RW::N; ++i) mbar_init(smem_addr(&bar_raw[i]), 1);
     abort_flag = 0;
     mbar_init_fence();
     if (XTMA) {
@@ -235,12 +283,12 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_contract_kernel(
   const uint32_t raw0 = sbase + C_CONV * C_CONV_BYTES;
   const int nsub = (nch + p.sub_ks - 1) / p.sub_ks;
 
-  if (warp >= 5) {
+  if (warp > MMA_WARP) {
     const int q = warp & 3;             // TMEM lane quadrant: rows 32q .. 32q + 31
     const uint32_t tile = sbase + RW::TILES + q * C_TILE_BYTES;
-    const int e0 = eb * ROWS + 32 * q;  // first row of the quadrant
-    float2* part = p.part + ((long long)s * p.n_freq + l) * p.NE * p.NE;
-    const int rsub = lane >> 4, csub = lane & 15;  // read-back position in a tile
+    float2* part = p.part + ((long long)s * p.n_freq + l) * p.NE * p.NE +
+                   (long long)er0 * p.NE + jr0;
+    const int rsub = lane >> 3, csub = lane & 7;  // read-back position in a tile
     for (int sub = 0; sub < nsub; ++sub) {
       const int b = sub & 1;
       const bool ok = mbar_wait(smem_addr(&bar_done[b]), (sub >> 1) & 1, &abort_flag, p.err,
@@ -248,33 +296,35 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_contract_kernel(
       fence_after_sync();
       const uint32_t lane_addr = tmem + ((uint32_t)(32 * q) << 16) + 256u * b;
 #pragma unroll 1
-      for (int cb = 0; cb < ROWS / 16; ++cb) {
-        uint32_t re[16], im[16];
-        tmem_ld16(lane_addr + 16 * cb, re);
-        tmem_ld16(lane_addr + ROWS + 16 * cb, im);
+      for (int cb = 0; cb < nbr / 8; ++cb) {
+        uint32_t re[8], im[8];
+        tmem_ld8(lane_addr + 8 * cb, re);
+        tmem_ld8(lane_addr + nbr + 8 * cb, im);
         tmem_wait_ld();
-        // this lane's row (32q + lane), columns 16 cb .. 16 cb + 15
+        // this lane's row (32q + lane), columns 8 cb .. 8 cb + 7
 #pragma unroll
-        for (int k = 0; k < 16; ++k)
+        for (int k = 0; k < 8; ++k)
           sts64(tile + (uint32_t)((lane * C_TILE_STRIDE + k) * 8), __uint_as_float(re[k]),
                 __uint_as_float(im[k]));
         __syncwarp();
-        const int jj = jb * ROWS + 16 * cb + csub;
-#pragma unroll 4
-        for (int ii = 0; ii < 16; ++ii) {
-          const int rr = 2 * ii + rsub;
-          const int e = e0 + rr;
+        const int jj = 8 * cb + csub;
+        float2 o[8];
+#pragma unroll
+        for (int ii = 0; ii < 8; ++ii) {
+          const int e = 32 * q + 4 * ii + rsub;
+          o[ii] = (sub > 0 && e < ne && jj < nj) ? part[(long long)e * p.NE + jj]
+                                                 : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int ii = 0; ii < 8; ++ii) {
+          const int rr = 4 * ii + rsub, e = 32 * q + rr;
           const float2 t = lds64(tile + (uint32_t)((rr * C_TILE_STRIDE + csub) * 8));
-          if (e < p.NE && jj < p.NE) {
-            float2* dst = part + (long long)e * p.NE + jj;
-            float2 v = ok ? t : make_float2(0.f, 0.f);
-            if (sub > 0) {
-              const float2 o = *dst;
-              v.x += o.x;
-              v.y += o.y;
-            }
-            *dst = v;
+          float2 v = ok ? t : make_float2(0.f, 0.f);
+          if (sub > 0) {
+            v.x += o[ii].x;
+            v.y += o[ii].y;
           }
+          if (e < ne && jj < nj) part[(long long)e * p.NE + jj] = v;
         }
         __syncwarp();
       }
@@ -282,30 +332,32 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_contract_kernel(
       mbar_arrive(smem_addr(&bar_freed[b]));
     }
     if (nch == 0) {
-      for (int rr = 0; rr < 32; ++rr) {
-        const int e = e0 + rr;
-        for (int jj = jb * ROWS + lane; jj < jb * ROWS + ROWS; jj += 32)
-          if (e < p.NE && jj < p.NE) part[(long long)e * p.NE + jj] = make_float2(0.f, 0.f);
-      }
+      for (int e = 32 * q; e < 32 * q + 32 && e < ne; ++e)
+        for (int jj = lane; jj < nj; jj += 32)
+          part[(long long)e * p.NE + jj] = make_float2(0.f, 0.f);
     }
-  } else if (warp < 4) {
-    const int r = tid;
+  } else if (warp < MMA_WARP) {
+    const int grp = tid / 128, r = tid % 128;
+    // the group's k-steps g = grp + GROUPS i, i < ni, through its RN raw stages
+    const int ni = (nch > grp) ? (nch - grp - 1) / GROUPS + 1 : 0;
     // raw fill: four lanes copy one row's 64-byte segment, so each warp
     // instruction reads eight rows in whole 32-byte sectors
     const int fq = r & 3;   // 16-byte piece of the segment
     const int fr = r >> 2;  // first row of this thread (rows fr + 32 k)
-    auto issue = [&](int g) {
-      if (g < nch) {
-        const long long n0 = n_begin + (long long)g * KS;
-        const uint32_t rb = raw0 + (uint32_t)((g % C_RAW) * C_RAW_BYTES);
+    auto issue = [&](int i) {
+      if (i < ni) {
+        const long long n0 = n_begin + (long long)(grp + GROUPS * i) * KS;
+        const int slot = grp * RN + i % RN;
+        const uint32_t rb = raw0 + (uint32_t)(slot * C_RAW_BYTES);
         if (XTMA) {
           // k-steps never straddle a chunk end (chunks are whole k-steps);
-          // rows e >= NE and pixels n >= N are outside the tensor: zero fill
+          // rows >= NE and pixels n >= N are outside the tensor (zero fill),
+          // rows of a tile past its tr are not used
           if (r == 0) {
-            const uint32_t bar = smem_addr(&bar_raw[g % C_RAW]);
+            const uint32_t bar = smem_addr(&bar_raw[slot]);
             mbar_arrive_expect_tx(bar, (uint32_t)CRawT<SHARED>::TX);
-            tma_load_3d(rb + C_RAW_X, &xmap, (int)(2 * n0), eb * ROWS, l, bar);
-            if (!same_rows) tma_load_3d(rb + C_RAW_Q, &qmap, (int)(2 * n0), jb * ROWS, l, bar);
+            tma_load_3d(rb + C_RAW_X, &xmap, (int)(2 * n0), er0, l, bar);
+            if (!same_rows) tma_load_3d(rb + C_RAW_Q, &qmap, (int)(2 * n0), jr0, l, bar);
           }
         } else {
           const long long n = n0 + 2 * fq;
@@ -313,40 +365,45 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_contract_kernel(
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             const int rr = fr + 32 * k;
-            const int er = eb * ROWS + rr, jr = jb * ROWS + rr;
-            const bool okx = okn && er < p.NE, okq = okn && jr < p.NE;
+            const bool okx = okn && rr < ne, okq = okn && rr < nj;
             cp_async16(rb + C_RAW_X + rr * C_RAWROW + 16 * fq,
-                       okx ? Xl + (long long)er * p.N + n : Xl, okx ? 16u : 0u);
+                       okx ? Xl + (long long)(er0 + rr) * p.N + n : Xl, okx ? 16u : 0u);
             if (!same_rows)
               cp_async16(rb + C_RAW_Q + rr * C_RAWROW + 16 * fq,
-                         okq ? Ql + (long long)jr * p.N + n : Ql, okq ? 16u : 0u);
+                         okq ? Ql + (long long)(jr0 + rr) * p.N + n : Ql, okq ? 16u : 0u);
           }
         }
         if (has_a && r < 4) {
           const long long n = n0 + 2 * r;
           const bool ok = n < n_end;
-          cp_async16(rb + C_RAW_A + 16 * r, ok ? p.a + n : p.a, ok ? 16u : 0u);
+          cp_async16(sbase + RW::AW + 64 * slot + 16 * r, ok ? p.a + n : p.a, ok ? 16u : 0u);
         }
       }
       cp_async_commit();
     };
+    // the raw stage of step i - 1 is free after step i's barrier
 #pragma unroll
-    for (int g = 0; g < C_RAW - 1; ++g) issue(g);
-    for (int g = 0; g < nch; ++g) {
+    for (int i = 0; i < (RN > 1 ? RN - 1 : 1); ++i) issue(i);
+    for (int i = 0; i < ni; ++i) {
+      const int g = grp + GROUPS * i;
+      const int slot = grp * RN + i % RN;
       if (XTMA)
-        mbar_wait(smem_addr(&bar_raw[g % C_RAW]), (g / C_RAW) & 1, &abort_flag, p.err,
-                  kErrWaitFull);
-      cp_async_wait<C_RAW - 2>();
-      bar_sync(1, 128);  // chunk g visible to all; everyone done with chunk g-1
-      issue(g + C_RAW - 1);
+        mbar_wait(smem_addr(&bar_raw[slot]), (i / RN) & 1, &abort_flag, p.err, kErrWaitFull);
+      cp_async_wait<(RN > 1 ? RN - 2 : 0)>();
+      bar_sync(1 + grp, 128);  // step i visible to the group; all done with step i - 1
+      if (RN > 1) issue(i + RN - 1);
       const int cs = g % C_CONV;
       mbar_wait(smem_addr(&bar_empty[cs]), ((g / C_CONV) & 1) ^ 1, &abort_flag, p.err,
                 kErrWaitEmpty);
-      const uint32_t rb = raw0 + (uint32_t)((g % C_RAW) * C_RAW_BYTES);
+      const uint32_t rb = raw0 + (uint32_t)(slot * C_RAW_BYTES);
+      const uint32_t ra = sbase + RW::AW + 64 * slot;
       const uint32_t cb = sbase + (uint32_t)(cs * C_CONV_BYTES);
-      const uint32_t bhi = cb + 4 * PLANE, blo = bhi + BPLANE;
+      const uint32_t bhi = cb + 4 * PLANE, blo = bhi + bplane((uint32_t)nbr);
+      // warps whose rows are all padding have nothing to convert
+      const bool work = r < ne || r < nbr;
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
+        if (!work) break;
         float2 x[4], q[4];
         // chunks 2 half and 2 half + 1 of row r (swizzled when TMA filled)
         const uint32_t o0 = XTMA ? swz64(r, 2 * half) : (uint32_t)(r * C_RAWROW + 32 * half);
@@ -367,8 +424,8 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_contract_kernel(
           q[2] = make_float2(u1.x, u1.y); q[3] = make_float2(u1.z, u1.w);
         }
         if (has_a) {
-          const float4 u0 = lds128(rb + C_RAW_A + 32 * half);
-          const float4 u1 = lds128(rb + C_RAW_A + 32 * half + 16);
+          const float4 u0 = lds128(ra + 32 * half);
+          const float4 u1 = lds128(ra + 32 * half + 16);
           const float2 av[4] = {make_float2(u0.x, u0.y), make_float2(u0.z, u0.w),
                                 make_float2(u1.x, u1.y), make_float2(u1.z, u1.w)};
 #pragma unroll
@@ -380,45 +437,57 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_contract_kernel(
         const float xi[4] = {x[0].y, x[1].y, x[2].y, x[3].y};
         const float qr[4] = {q[0].x, q[1].x, q[2].x, q[3].x};
         const float qi[4] = {q[0].y, q[1].y, q[2].y, q[3].y};
-        put_a(cb + 0 * PLANE, cb + 1 * PLANE, half, r, xr);
-        put_a(cb + 2 * PLANE, cb + 3 * PLANE, half, r, xi);
-        put_b(bhi, blo, half, r, qr, qi);
+        if (r < ne) {
+          put_a(cb + 0 * PLANE, cb + 1 * PLANE, half, r, xr);
+          put_a(cb + 2 * PLANE, cb + 3 * PLANE, half, r, xi);
+        }
+        if (r < nbr) put_b(bhi, blo, half, r, nbr, qr, qi);
       }
       fence_proxy_async();
       if (!(p.stall && g == 0)) mbar_arrive(smem_addr(&bar_full[cs]));
+      if (RN == 1) {
+        bar_sync(1 + grp, 128);  // the group's only raw stage is free
+        issue(i + 1);
+      }
     }
     cp_async_wait<0>();
     if (XTMA && r == 0 && abort_flag) {
       // copies issued before a wait gave up may still land in this CTA's
       // shared memory: wait (bounded) for the last one of every raw stage
-      for (int i = 0; i < C_RAW && i < nch; ++i) {
-        const int g = nch - 1 - ((nch - 1 - i) % C_RAW);
-        mbar_wait_drain(smem_addr(&bar_raw[g % C_RAW]), (g / C_RAW) & 1, p.err, kErrWaitDrain);
+      for (int k = 0; k < RN && k < ni; ++k) {
+        const int i = ni - 1 - ((ni - 1 - k) % RN);
+        mbar_wait_drain(smem_addr(&bar_raw[grp * RN + i % RN]), (i / RN) & 1, p.err,
+                        kErrWaitDrain);
       }
     }
   } else {
+    int cs = 0, use = 0, ks = 0, sub = 0;  // stage, its use, k-step of the sub-chunk
+    const KStep step((uint32_t)nbr);
     for (int g = 0; g < nch; ++g) {
-      const int cs = g % C_CONV;
-      const int sub = g / p.sub_ks, b = sub & 1;
-      if (g % p.sub_ks == 0 && sub >= 2) {
+      const int b = sub & 1;
+      if (ks == 0 && sub >= 2) {
         // buffer b is free once sub-chunk sub - 2 has been drained
         mbar_wait(smem_addr(&bar_freed[b]), ((sub - 2) >> 1) & 1, &abort_flag, p.err,
                   kErrWaitEmpty);
         fence_after_sync();
       }
-      const bool ok = mbar_wait(smem_addr(&bar_full[cs]), (g / C_CONV) & 1, &abort_flag,
-                                p.err, kErrWaitFull);
+      const bool ok = mbar_wait(smem_addr(&bar_full[cs]), use & 1, &abort_flag, p.err,
+                                kErrWaitFull);
       fence_after_sync();
-      if (lane == 0 && ok) {
-        const uint32_t cb = sbase + (uint32_t)(cs * C_CONV_BYTES);
-        issue_kstep(tmem + 256u * b, cb, cb + 4 * PLANE, g % p.sub_ks == 0);
-        commit(smem_addr(&bar_empty[cs]));
+      const bool last = ks == p.sub_ks - 1 || g == nch - 1;
+      if (elect_one()) {
+        if (ok) {
+          const uint32_t cb = sbase + (uint32_t)(cs * C_CONV_BYTES);
+          step.issue(tmem + 256u * b, cb, cb + 4 * PLANE, ks == 0);
+          commit(smem_addr(&bar_empty[cs]));
+        }
+        if (last) commit(smem_addr(&bar_done[b]));
       }
-      if (lane == 0 && ((g + 1) % p.sub_ks == 0 || g == nch - 1))
-        commit(smem_addr(&bar_done[b]));
       __syncwarp();
+      if (++cs == C_CONV) { cs = 0; ++use; }
+      if (last) { ks = 0; ++sub; } else { ++ks; }
     }
-    if (lane == 0) commit(smem_addr(&bar_final));  // after every MMA of this CTA
+    if (elect_one()) commit(smem_addr(&bar_final));  // after every MMA of this CTA
   }
   fence_before_sync();
   __syncthreads();
@@ -434,11 +503,12 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_contract_kernel(
 
 // ---------------------------------------------------------------------------
 // J^H: persistent CTAs over units (frequency l, element tile eb, tile of 128
-// pixels).  Per unit the accumulator holds W[n][e] (128 pixels x [128 Re |
-// 128 Im]); two accumulators alternate between units, and four epilogue
+// pixels).  Per unit the accumulator holds W[n][e] (128 pixels x [nbr Re |
+// nbr Im], nbr the tile's elements rounded up to 8); two accumulators
+// alternate between units, and four epilogue
 // warps form s_l sum_e conj(X[e][n]) W[e][n] into zpart[l][eb][n] (FUSED) or
 // write W itself while the MMAs of the next unit proceed.
-constexpr int M_CONV = 3, M_RAW = 6;
+constexpr int M_CONV = 4, M_RN = 2, M_RAW = GROUPS * M_RN;
 constexpr int M_RAW_BYTES = KS * ROWS * 8;               // [8 j][128 n] complex
 constexpr int M_A_BYTES = 4 * PLANE;
 constexpr int M_B_BYTES = 2 * BPLANE;                    // one k-step of B hi + lo
@@ -463,6 +533,11 @@ struct JhArgs {
 // XTMA: the raw tiles of the mixed operand (8 rows j x 128 pixels, one box)
 // arrive by TMA tensor copies issued by one producer thread and completing
 // on bar_raw; otherwise every producer copies its part with cp.async.
+__host__ __device__ __forceinline__ int jh_rows(int NE, int eb) {
+  const int n = NE - eb * ROWS;
+  return round8(n < ROWS ? n : ROWS);
+}
+
 template <bool FUSED, bool XTMA>
 __global__ void __launch_bounds__(C_THREADS, 1) tc_jh_kernel(JhArgs p,
                                                              const __grid_constant__ CUtensorMap xmap) {
@@ -512,7 +587,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_jh_kernel(JhArgs p,
     l = u / (p.npb * p.nbe);
   };
 
-  if (warp >= 5) {
+  if (warp > MMA_WARP) {
     // epilogue warps: TMEM lane = pixel 32 q + lane of the unit's tile
     const int q = warp & 3;
     const int r = 32 * q + lane;
@@ -529,11 +604,14 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_jh_kernel(JhArgs p,
       const long long n = (long long)pb * ROWS + r;
       const bool nv = n < p.N;
       float zx = 0.f, zy = 0.f;
+      const int nbr = jh_rows(p.NE, eb);
 #pragma unroll 1
-      for (int ec = 0; ec < ROWS / 32; ++ec) {
+      for (int ec = 0; 32 * ec < nbr; ++ec) {
+        // (columns past nbr hold other values of the accumulator; rows e >= NE
+        // are skipped below)
         uint32_t wr[32], wi[32];
         tmem_ld32(lane_addr + (uint32_t)(32 * ec), wr);
-        tmem_ld32(lane_addr + (uint32_t)(ROWS + 32 * ec), wi);
+        tmem_ld32(lane_addr + (uint32_t)(nbr + 32 * ec), wi);
         tmem_wait_ld();
         if constexpr (FUSED) {
 #pragma unroll
@@ -565,18 +643,22 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_jh_kernel(JhArgs p,
       fence_before_sync();  // the TMEM reads precede the buffer's next MMAs
       mbar_arrive(smem_addr(&bar_freed[b]));
     }
-  } else if (warp < 4) {
-    const int r = tid;
-    auto issue = [&](int g) {
-      if (g < nchunks) {
+  } else if (warp < MMA_WARP) {
+    const int grp = tid / 128, r = tid % 128;
+    // the group's k-steps g = grp + GROUPS i, i < ni, through its M_RN raw stages
+    const int ni = (nchunks > grp) ? (nchunks - grp - 1) / GROUPS + 1 : 0;
+    auto issue = [&](int i) {
+      if (i < ni) {
+        const int g = grp + GROUPS * i;
         int l, eb, pb;
         unit_of(g / p.nks, l, eb, pb);
         const int ks = g % p.nks;
-        const uint32_t rb = raw0 + (uint32_t)((g % M_RAW) * M_RAW_BYTES);
+        const int slot = grp * M_RN + i % M_RN;
+        const uint32_t rb = raw0 + (uint32_t)(slot * M_RAW_BYTES);
         if (XTMA) {
           // rows j >= NE and pixels n >= N are outside the tensor: zero fill
           if (r == 0) {
-            const uint32_t bar = smem_addr(&bar_raw[g % M_RAW]);
+            const uint32_t bar = smem_addr(&bar_raw[slot]);
             mbar_arrive_expect_tx(bar, M_RAW_BYTES);
             tma_load_3d(rb, &xmap, 2 * pb * ROWS, ks * KS, l, bar);
           }
@@ -584,8 +666,8 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_jh_kernel(JhArgs p,
           const float2* Xl = p.X + (long long)l * p.NE * p.N;
 #pragma unroll
           for (int k = 0; k < (KS * ROWS / 2) / 128; ++k) {
-            const int i = r + 128 * k;
-            const int jj = i / (ROWS / 2), pr = i % (ROWS / 2);
+            const int q = r + 128 * k;
+            const int jj = q / (ROWS / 2), pr = q % (ROWS / 2);
             const int jrow = ks * KS + jj;
             const long long n = (long long)pb * ROWS + 2 * pr;
             const bool ok = (jrow < p.NE) && (n < p.N);
@@ -597,15 +679,16 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_jh_kernel(JhArgs p,
       if (!XTMA) cp_async_commit();
     };
 #pragma unroll
-    for (int g = 0; g < M_RAW - 1; ++g) issue(g);
-    for (int g = 0; g < nchunks; ++g) {
+    for (int i = 0; i < M_RN - 1; ++i) issue(i);
+    for (int i = 0; i < ni; ++i) {
+      const int g = grp + GROUPS * i;
+      const int slot = grp * M_RN + i % M_RN;
       if (XTMA)
-        mbar_wait(smem_addr(&bar_raw[g % M_RAW]), (g / M_RAW) & 1, &abort_flag, p.err,
-                  kErrWaitFull);
+        mbar_wait(smem_addr(&bar_raw[slot]), (i / M_RN) & 1, &abort_flag, p.err, kErrWaitFull);
       else
-        cp_async_wait<M_RAW - 2>();
-      bar_sync(1, 128);
-      issue(g + M_RAW - 1);
+        cp_async_wait<M_RN - 2>();
+      bar_sync(1 + grp, 128);
+      issue(i + M_RN - 1);
       const int kunit = g / p.nks, ks = g % p.nks;
       int l, eb, pb;
       unit_of(kunit, l, eb, pb);
@@ -615,12 +698,13 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_jh_kernel(JhArgs p,
       const uint32_t cb = sbase + (uint32_t)(cs * M_CONV_BYTES);
       if (r == 0) {
         const uint32_t fb = smem_addr(&bar_full[cs]);
-        mbar_arrive_expect_tx(fb, M_B_BYTES);
+        const uint32_t bytes = 2 * bplane((uint32_t)jh_rows(p.NE, eb));
+        mbar_arrive_expect_tx(fb, bytes);
         const float* src =
             p.bops + ((((long long)l * p.nbe + eb) * p.nks + ks) * (long long)(M_B_BYTES / 4));
-        bulk_g2s(cb + M_A_BYTES, src, M_B_BYTES, fb);
+        bulk_g2s(cb + M_A_BYTES, src, bytes, fb);
       }
-      const uint32_t rb = raw0 + (uint32_t)((g % M_RAW) * M_RAW_BYTES);
+      const uint32_t rb = raw0 + (uint32_t)(slot * M_RAW_BYTES);
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
         float re[4], im[4];
@@ -641,32 +725,45 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_jh_kernel(JhArgs p,
     } else if (r == 0 && abort_flag) {
       // copies issued before a wait gave up may still land in this CTA's
       // shared memory: wait (bounded) for the last one of every raw stage
-      for (int i = 0; i < M_RAW && i < nchunks; ++i) {
-        const int g = nchunks - 1 - ((nchunks - 1 - i) % M_RAW);
-        mbar_wait_drain(smem_addr(&bar_raw[g % M_RAW]), (g / M_RAW) & 1, p.err, kErrWaitDrain);
+      for (int k = 0; k < M_RN && k < ni; ++k) {
+        const int i = ni - 1 - ((ni - 1 - k) % M_RN);
+        mbar_wait_drain(smem_addr(&bar_raw[grp * M_RN + i % M_RN]), (i / M_RN) & 1, p.err,
+                        kErrWaitDrain);
       }
     }
   } else {
+    int cs = 0, use = 0, ks = 0, kunit = 0;
+    KStep step(8);
     for (int g = 0; g < nchunks; ++g) {
-      const int cs = g % M_CONV, ks = g % p.nks, kunit = g / p.nks, b = kunit & 1;
-      if (ks == 0 && kunit >= 2) {
-        // buffer b is free once unit kunit - 2 has been read out
-        mbar_wait(smem_addr(&bar_freed[b]), ((kunit - 2) >> 1) & 1, &abort_flag, p.err,
-                  kErrWaitEmpty);
-        fence_after_sync();
+      const int b = kunit & 1;
+      if (ks == 0) {
+        int l, eb, pb;
+        unit_of(kunit, l, eb, pb);
+        step = KStep((uint32_t)jh_rows(p.NE, eb));
+        if (kunit >= 2) {
+          // buffer b is free once unit kunit - 2 has been read out
+          mbar_wait(smem_addr(&bar_freed[b]), ((kunit - 2) >> 1) & 1, &abort_flag, p.err,
+                    kErrWaitEmpty);
+          fence_after_sync();
+        }
       }
-      const bool ok = mbar_wait(smem_addr(&bar_full[cs]), (g / M_CONV) & 1, &abort_flag,
-                                p.err, kErrWaitFull);
+      const bool ok = mbar_wait(smem_addr(&bar_full[cs]), use & 1, &abort_flag, p.err,
+                                kErrWaitFull);
       fence_after_sync();
-      if (lane == 0 && ok) {
-        const uint32_t cb = sbase + (uint32_t)(cs * M_CONV_BYTES);
-        issue_kstep(tmem + 256u * b, cb, cb + M_A_BYTES, ks == 0);
-        commit(smem_addr(&bar_empty[cs]));
+      const bool last = ks == p.nks - 1;
+      if (elect_one()) {
+        if (ok) {
+          const uint32_t cb = sbase + (uint32_t)(cs * M_CONV_BYTES);
+          step.issue(tmem + 256u * b, cb, cb + M_A_BYTES, ks == 0);
+          commit(smem_addr(&bar_empty[cs]));
+        }
+        if (last) commit(smem_addr(&bar_done[b]));
       }
-      if (lane == 0 && ks == p.nks - 1) commit(smem_addr(&bar_done[b]));
       __syncwarp();
+      if (++cs == M_CONV) { cs = 0; ++use; }
+      if (last) { ks = 0; ++kunit; } else { ++ks; }
     }
-    if (lane == 0) commit(smem_addr(&bar_final));  // after every MMA of this CTA
+    if (elect_one()) commit(smem_addr(&bar_final));  // after every MMA of this CTA
   }
   fence_before_sync();
   __syncthreads();
@@ -691,7 +788,9 @@ __global__ void tc_jh_bops_kernel(const V* __restrict__ y, float* __restrict__ b
     const int hl = rem / (2 * BROWS), half = (rem / BROWS) % 2, row = rem % BROWS;
     const int ks = (int)(blk % nks), eb = (int)((blk / nks) % nbe);
     const long long l = blk / ((long long)nks * nbe);
-    const int e = eb * ROWS + row % ROWS, part = row / ROWS;
+    const int nbr = jh_rows(NE, eb);
+    const int e = eb * ROWS + row % nbr, part = row / nbr;
+    if (part > 2) continue;  // past the tile's three blocks
     float v[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -704,8 +803,8 @@ __global__ void tc_jh_bops_kernel(const V* __restrict__ y, float* __restrict__ b
       const float hi = tc::to_tf32((float)x);
       v[k] = hl == 0 ? hi : tc::to_tf32((float)(x - (double)hi));
     }
-    float4* dst = (float4*)(bops + blk * (M_B_BYTES / 4) + hl * (BPLANE / 4) +
-                            half * (16 * BROWS / 4) + 4 * row);
+    float4* dst = (float4*)(bops + blk * (M_B_BYTES / 4) + hl * (24 * nbr) + half * (12 * nbr) +
+                            4 * row);
     *dst = make_float4(v[0], v[1], v[2], v[3]);
   }
 }
@@ -809,7 +908,8 @@ int tc_contract_partials(fwi_ctx* c, const float2* X, const float2* a, const flo
   const long long chunk_ks = chunk / KS;
   const long long nsub = (chunk_ks + 63) / 64;
   const int sub_ks = (int)((chunk_ks + nsub - 1) / nsub);
-  ContractArgs args{X, Q, a, part, c->tc_err, c->N, chunk, c->n_elem, c->n_freq, sub_ks,
+  const int tr = round8((c->n_elem + nbe - 1) / nbe);
+  ContractArgs args{X, Q, a, part, c->tc_err, c->N, chunk, c->n_elem, c->n_freq, tr, sub_ks,
                     c->tc_stall};
   c->tc_stall = 0;  // one launch
   dim3 grid(split, nbe * nbe, c->n_freq);
