@@ -471,11 +471,11 @@ typedef struct fwi_tuning {
                            same arithmetic on the same values: results agree
                            to FP32 rounding. */
   int col_spectrum_stage; /* 1 (default): with col_tma, the convolution also
-                           stages its kernel-spectrum tiles with TMA where
-                           they fit (half the column's rows, the spectrum
-                           being even; at most 256 rows); 0: the spectrum
-                           is read from global memory.  Results agree to
-                           FP32 rounding. */
+                           stages its kernel-spectrum tiles with TMA (half
+                           the column's rows, the spectrum being even; one
+                           column per thread: where they fit); 0: the
+                           spectrum is read from global memory.  Results
+                           agree to FP32 rounding. */
   int jac_tma;          /* 1 (default): the tensor-core pixel contractions
                            receive their raw FP32 operand tiles by TMA
                            tensor copies issued by one producer thread;
@@ -493,8 +493,8 @@ typedef struct fwi_tuning {
                            row_l2_prefetch).  Results agree to FP32
                            rounding. */
   int col_pairs;        /* 1 (default): the FP32 convolution pass, where its
-                           transform length is 16, 64 or 256 and its kernel
-                           spectrum is staged, computes two columns per
+                           kernel spectrum is staged (col_tma and
+                           col_spectrum_stage), computes two columns per
                            thread with packed f32x2 arithmetic on column
                            pairs; 0: one column per thread.  Results agree
                            to FP32 rounding. */

@@ -1,5 +1,4 @@
-// Convolution pass with two columns per thread (FP32; plans listed at
-// pair_plan: power-of-two DFTs, whole first DFTs per thread).
+// Convolution pass with two columns per thread (FP32, every transform length).
 //
 // The transforms are the four-step FFT of fft_core.cuh (forward FFT along
 // the column with the zero-padded half pruned, product with the kernel
@@ -15,11 +14,20 @@
 // products are formed as re*c - im*s with one rounding per product and per
 // sum, so results agree with the one-column kernel to FP32 rounding.
 //
-// The rest follows col_tma_kernel: persistent CTAs over the slot-fast item
-// order, the next item's input tile (and, where it fits, its kernel-spectrum
-// tile) staged by TMA into shared memory while the current item transforms,
-// bounded mbarrier waits with the same error codes.  Split plans share their
-// second DFTs over a lane pair, exchanging column pairs by warp shuffles.
+// Persistent CTAs hold one kernel-spectrum tile for a run of right-hand sides
+// and stage the next item's input tile by TMA while the current item transforms;
+// bounded mbarrier waits with the error codes of col_tma_kernel.
+//
+// What bounds it: FP32 issue and shared-memory traffic about equally (1024
+// points, 16 columns on one SM: 8,400 cycles of packed FP32 and 7,500 of
+// shared-memory accesses against 16,600 taken), with few warps to overlap the
+// two.  Cycles per 16 columns on one SM before (one column per thread, or lane
+// pairs sharing the 32-point DFTs of 512, and a spectrum tile copied or read
+// for every item) and now: 128: 2,370 -> 1,930; 192: 3,930 -> 2,980 (96^3:
+// 3,600 -> 2,560); 256: 3,430 -> 3,210; 320: 6,050 -> 5,210; 384: 8,500 ->
+// 5,990; 512: 9,310 -> 7,290; 640: 17,700 -> 12,250; 768: 17,000 -> 13,600;
+// 1024: 25,600 -> 16,600.  The 32-value plans at 168 registers and three CTAs per
+// SM, their spectrum read from L2, took 8,600 (512) to 21,000 (1024).
 #pragma once
 
 namespace fwi {
@@ -118,7 +126,21 @@ __device__ __forceinline__ PC pmul(PC z, u64 gr, u64 gi) {
   return {f2sub(f2mul(z.re, gr), f2mul(z.im, gi)), f2fma(z.re, gi, f2mul(z.im, gr))};
 }
 
-// In-register DFT of size R (a power of two), natural order, in place.
+// c * z, c the same for both columns
+__device__ __forceinline__ PC pscale(PC z, float c) {
+  const u64 cc = pk(c, c);
+  return {f2mul(z.re, cc), f2mul(z.im, cc)};
+}
+// a + c z
+__device__ __forceinline__ PC paxpy(float c, PC z, PC a) {
+  const u64 cc = pk(c, c);
+  return {f2fma(z.re, cc, a.re), f2fma(z.im, cc, a.im)};
+}
+// a +- i z
+__device__ __forceinline__ PC padd_i(PC a, PC z) { return {f2sub(a.re, z.im), f2add(a.im, z.re)}; }
+__device__ __forceinline__ PC psub_i(PC a, PC z) { return {f2add(a.re, z.im), f2sub(a.im, z.re)}; }
+
+// In-register DFT of size R (factors 2, 3, 4, 5), natural order, in place.
 template <int R, bool INV> struct PDft;
 template <bool INV> struct PDft<1, INV> {
   static __device__ __forceinline__ void run(PC*) {}
@@ -146,12 +168,40 @@ template <bool INV> struct PDft<4, INV> {
     }
   }
 };
+template <bool INV> struct PDft<3, INV> {
+  static __device__ __forceinline__ void run(PC* x) {
+    constexpr float s1 = INV ? 0.86602540378443864676f : -0.86602540378443864676f;
+    const PC sp = padd(x[1], x[2]), u = pscale(psub(x[1], x[2]), s1);
+    const PC t = paxpy(-0.5f, sp, x[0]);
+    x[0] = padd(x[0], sp);
+    x[1] = padd_i(t, u);
+    x[2] = psub_i(t, u);
+  }
+};
+template <bool INV> struct PDft<5, INV> {
+  static __device__ __forceinline__ void run(PC* x) {
+    // cosines and sines of 2 pi / 5 and 4 pi / 5
+    constexpr float c1 = 0.30901699437494742410f, c2 = -0.80901699437494742410f;
+    constexpr float s1 = INV ? 0.95105651629515357212f : -0.95105651629515357212f;
+    constexpr float s2 = INV ? 0.58778525229247312917f : -0.58778525229247312917f;
+    const PC a = x[0];
+    const PC p1 = padd(x[1], x[4]), m1 = psub(x[1], x[4]);
+    const PC p2 = padd(x[2], x[3]), m2 = psub(x[2], x[3]);
+    const PC t1 = paxpy(c2, p2, paxpy(c1, p1, a)), t2 = paxpy(c1, p2, paxpy(c2, p1, a));
+    const PC u1 = paxpy(s2, m2, pscale(m1, s1)), u2 = paxpy(-s1, m2, pscale(m1, s2));
+    x[0] = padd(a, padd(p1, p2));
+    x[1] = padd_i(t1, u1);
+    x[4] = psub_i(t1, u1);
+    x[2] = padd_i(t2, u2);
+    x[3] = psub_i(t2, u2);
+  }
+};
 // R = A * B: A-point DFTs over n1 (n = B n1 + n2), twiddle w_R^{n2 k1},
 // B-point DFTs over n2; output index k = k1 + A k2.
 template <int R, bool INV> struct PDft {
   static constexpr int A = first_factor(R);
   static constexpr int B = R / A;
-  static_assert((R & (R - 1)) == 0 && A * B == R && B > 1, "power-of-two sizes only");
+  static_assert(A * B == R && B > 1, "factors 2, 3, 4, 5 only");
   static __device__ __forceinline__ void run(PC* x) {
     PC y[R];
     SFor<B>::run([&](auto n2c) {
@@ -214,150 +264,136 @@ template <int R, bool INV> struct PDftHalfOut {
   }
 };
 
-// Exchange of a pair with the partner lane of a split DFT (16 lanes away).
-__device__ __forceinline__ PC shfl_pc(PC a) {
-  float x0, x1, y0, y1;
-  upk(a.re, x0, x1);
-  upk(a.im, y0, y1);
-  x0 = __shfl_xor_sync(0xffffffffu, x0, 16);
-  x1 = __shfl_xor_sync(0xffffffffu, x1, 16);
-  y0 = __shfl_xor_sync(0xffffffffu, y0, 16);
-  y1 = __shfl_xor_sync(0xffffffffu, y1, 16);
-  return {pk(x0, x1), pk(y0, y1)};
-}
-// z * (h w + (1 - h)) with w = w_R^J (conjugated for INV): lane h = 0 keeps
-// z, lane 1 gets z w (hf = h, hc = 1 - h are exactly 0 or 1)
-template <int J, int R, bool INV>
-__device__ __forceinline__ PC plane_twiddle(PC z, float hf, float hc) {
-  constexpr int q = tw_quarter(J, R);
-  if constexpr (q == 0) {
-    return z;
-  } else {
-    constexpr double wr = q == 2 ? -1.0 : (q == 1 || q == 3) ? 0.0 : tw_re(J, R);
-    constexpr double wf = q == 1 ? -1.0 : q == 3 ? 1.0 : q == 2 ? 0.0 : tw_im(J, R);
-    constexpr double wi = INV ? -wf : wf;
-    const float av = hf * (float)wr + hc;
-    const float bv = hf * (float)wi;
-    return ptw_tab(z, pk(av, av), pk(bv, bv));
-  }
-}
-// R = 2Q point DFT over a lane pair (lanes 16 apart).  split: lane h holds
-// x[2m + h] (m < Q) and ends with X[k + Q h] (k < Q).  isplit: lane h holds
-// X[k + Q h] and ends with x[2m + h] (unnormalised).
-template <int Q, bool INV> __device__ __forceinline__ void psplit_dft(PC* u, int h) {
-  PDft<Q, INV>::run(u);
-  const float hf = (float)h, hc = (float)(1 - h), sg = (float)(1 - 2 * h);
-  const u64 sgp = pk(sg, sg);
-  SFor<Q>::run([&](auto kc) {
-    constexpr int k = decltype(kc)::value;
-    const PC v = plane_twiddle<k, 2 * Q, INV>(u[k], hf, hc);
-    const PC o = shfl_pc(v);
-    u[k] = {f2fma(sgp, v.re, o.re), f2fma(sgp, v.im, o.im)};
-  });
-}
-template <int Q, bool INV> __device__ __forceinline__ void psplit_idft(PC* u, int h) {
-  const float hf = (float)h, hc = (float)(1 - h), sg = (float)(1 - 2 * h);
-  const u64 sgp = pk(sg, sg);
-  SFor<Q>::run([&](auto kc) {
-    constexpr int k = decltype(kc)::value;
-    const PC own = u[k];
-    const PC o = shfl_pc(own);
-    const PC z = {f2fma(sgp, own.re, o.re), f2fma(sgp, own.im, o.im)};
-    u[k] = plane_twiddle<k, 2 * Q, INV>(z, hf, hc);
-  });
-  PDft<Q, INV>::run(u);
-}
-
 }  // namespace pair
 
-constexpr bool pow2_at_least(int r, int m) { return r >= m && (r & (r - 1)) == 0; }
+// Line plans of the two-column kernel: R1 x R2 with TL threads per column pair
+// (thread t owns n2 = t + i TL in phases A and D, k1 = t + i TL in B and C).
+template <int L> struct PairPlanFor;
+template <> struct PairPlanFor<16> { using type = Plan<16, 4, 4, 4>; };
+template <> struct PairPlanFor<32> { using type = Plan<32, 4, 8, 4>; };
+template <> struct PairPlanFor<64> { using type = Plan<64, 8, 8, 8>; };
+template <> struct PairPlanFor<128> { using type = Plan<128, 16, 8, 8>; };
+template <> struct PairPlanFor<192> { using type = Plan<192, 12, 16, 16>; };
+template <> struct PairPlanFor<256> { using type = Plan<256, 16, 16, 16>; };
+template <> struct PairPlanFor<320> { using type = Plan<320, 20, 16, 20>; };
+template <> struct PairPlanFor<384> { using type = Plan<384, 24, 16, 24>; };
+template <> struct PairPlanFor<512> { using type = Plan<512, 32, 16, 16>; };
+template <> struct PairPlanFor<640> { using type = Plan<640, 32, 20, 32>; };
+template <> struct PairPlanFor<768> { using type = Plan<768, 32, 24, 32>; };
+template <> struct PairPlanFor<1024> { using type = Plan<1024, 32, 32, 32>; };
 
-// Plans the two-column kernel covers: unsplit plans with one thread per n2
-// and per k1 (R1 = R2 = TL), and split plans whose first DFTs are whole
-// (S1 = 1) and whose second DFTs are shared by a lane pair (S2 = 2); all
-// DFT sizes powers of two.
-template <class P> constexpr bool pair_plan() {
-  if constexpr (PlanTraits<P>::split) {
-    return P::S1 == 1 && P::S2 == 2 && pow2_at_least(P::R1, 4) && pow2_at_least(P::Q2, 2);
-  } else {
-    return P::R1 == P::TL && P::R2 == P::TL && pow2_at_least(P::R1, 4);
-  }
-}
-
-// Shared memory (bytes from the 128-byte aligned base): exchange L x TC/2
-// pairs (16 bytes each) | input staging rows_in x TC | spectrum staging
-// (L/2 + 1) x TC (GS only) | pair twiddle table L x (c, c, s, s) | two
-// mbarriers and the abort flag.
-template <int L, int TC> struct ColPairSmem {
-  static constexpr int G_ROWS = L / 2 + 1;
-  static constexpr size_t bytes(int rows_in, bool gs) {
-    return ((size_t)L * TC + (size_t)rows_in * TC + (gs ? (size_t)G_ROWS * TC : 0)) *
-               sizeof(float2) +
-           (size_t)L * sizeof(float4) + 32 + 128;
+// Shared memory (bytes from the 128-byte aligned base): exchange, R2 rows of
+// R1 (+ 1 for tiles under 8 pairs, whose rows would otherwise start in the same
+// banks) x NP pairs of 16 bytes | input staging rows_in x TC (unless it lies in
+// the exchange) | kernel-spectrum tile, rows 0..L/2 in GBOX boxes of at most 256
+// rows | twiddle table L | two mbarriers and the abort flag.
+// ALIAS: the input staging lies inside the exchange buffer (free until every
+// thread holds its samples) where a separate one would leave one CTA per SM;
+// the next item's copy then starts when the inverse transforms have read the
+// exchange, behind an L2 prefetch.
+template <class P, int TC> struct ColPairSmem {
+  static constexpr int GBOX = (P::L / 2 + 1 + 255) / 256;
+  // (several boxes: whole 128-byte units each, as TMA destinations have to be;
+  // the rows past L/2 + 1 are spectrum rows nobody reads)
+  static constexpr int G_BOX_ROWS =
+      GBOX == 1 ? P::L / 2 + 1 : ((P::L / 2 + 1 + GBOX - 1) / GBOX + 3) / 4 * 4;
+  static constexpr int G_ROWS = GBOX * G_BOX_ROWS;
+  static constexpr int R1P = P::R1 + (TC < 16 ? 1 : 0);
+  static constexpr bool ALIAS = (P::L == 512 && TC == 16) || P::L == 1024;
+  static constexpr int ROW = TC * (int)sizeof(float2);
+  static_assert(P::R2 * R1P * ROW % 128 == 0 && P::L / 2 * ROW % 128 == 0 &&
+                (GBOX == 1 || G_BOX_ROWS * ROW % 128 == 0) && G_ROWS <= P::L &&
+                G_BOX_ROWS <= 256, "TMA destinations and boxes");
+  static constexpr size_t bytes(int rows_in) {
+    return ((size_t)P::R2 * R1P * TC + (ALIAS ? 0 : (size_t)rows_in * TC) +
+            (size_t)G_ROWS * TC + (size_t)P::L) * sizeof(float2) + 32 + 128;
   }
 };
 
-// GS: the kernel spectrum tile of each item is staged by TMA (rows 0..L/2);
-// otherwise each thread reads its spectrum pairs from global memory (L2).
-// Registers: 168 keeps three 128-thread CTAs per SM (the shared memory of
-// the 256-point convolution holds three as well); 256-thread CTAs get 128
-// (two per SM).
-constexpr int pair_regs(int threads) { return threads > 128 ? 128 : 168; }
-template <class P, int TC, bool GS>
-__global__ void __launch_bounds__(TC / 2 * P::TL,
-                                  blocks_for_regs(TC / 2 * P::TL, pair_regs(TC / 2 * P::TL)))
+// CTAs that take adjacent column tiles of the same right-hand side together.
+__host__ __device__ constexpr unsigned pair_group(unsigned ntile) {
+  return ntile % 8 == 0 ? 8u : ntile % 4 == 0 ? 4u : ntile % 2 == 0 ? 2u : 1u;
+}
+
+// Work order: the (tile group, right-hand side) items, right-hand side fastest,
+// are cut into one contiguous range per group of pair_group() CTAs, each of
+// which takes one tile of the group.  A CTA so keeps the kernel-spectrum tile
+// of one (tile, frequency) in shared memory for as many right-hand sides as its
+// range holds, instead of copying it from L2 for every item (as many bytes as
+// the input), and the group reads each right-hand side's rows in runs of up to
+// 1 KB.  Registers: a pair value takes four; the plans of up to 24 values a
+// thread run at 168 (three 128-thread CTAs per SM), those of 32 at up to 255.
+template <class P> constexpr int pair_blocks(int threads) {
+  return P::E > 24 ? 2 * (128 / threads > 1 ? 128 / threads : 1) : blocks_for_regs(threads, 168);
+}
+template <class P, int TC>
+__global__ void __launch_bounds__(TC / 2 * P::TL, pair_blocks<P>(TC / 2 * P::TL))
 col_pair_kernel(const ColArgs<float> a, const __grid_constant__ CUtensorMap map,
                 const __grid_constant__ CUtensorMap gmap, int rows_in, int nbox) {
   using namespace pair;
-  static_assert(pair_plan<P>(), "two-column plan");
-  constexpr bool SPLIT = PlanTraits<P>::split;
   constexpr int NP = TC / 2;  // column pairs per tile
-  constexpr int GP = 32 / NP;  // consecutive line threads per warp
-  constexpr int R1 = P::R1, R2 = P::R2, H1 = P::H1;
-  constexpr int NB = PlanTraits<P>::MB;  // phase-B values per thread (R2, or Q2 split)
-  constexpr int G_ROWS = ColPairSmem<P::L, TC>::G_ROWS;
+  constexpr int R1 = P::R1, R2 = P::R2, H1 = P::H1, C1 = P::C1, C3 = P::C3, TL = P::TL;
+  using SM = ColPairSmem<P, TC>;
+  constexpr int R1P = SM::R1P;
+  constexpr bool ALIAS = SM::ALIAS;
   extern __shared__ __align__(16) unsigned char smraw[];
   const uint32_t base_pad = (128u - (tc::smem_addr(smraw) & 127u)) & 127u;
-  float4* ex = reinterpret_cast<float4*>(smraw + base_pad);        // exchange, L x NP
-  float2* stg = reinterpret_cast<float2*>(ex + P::L * NP);         // input staging
-  float2* gst = stg + rows_in * TC;                                // spectrum staging
-  float4* twp = reinterpret_cast<float4*>(gst + (GS ? G_ROWS * TC : 0));  // pair twiddles
-  uint64_t* bar = reinterpret_cast<uint64_t*>(twp + P::L);         // [0] input, [1] spectrum
+  float4* ex = reinterpret_cast<float4*>(smraw + base_pad);        // exchange
+  float2* ex_end = reinterpret_cast<float2*>(ex + R2 * R1P * NP);
+  float2* stg = ALIAS ? reinterpret_cast<float2*>(ex) : ex_end;    // input staging
+  float2* gst = ex_end + (ALIAS ? 0 : rows_in * TC);               // spectrum staging
+  float2* tws = gst + SM::G_ROWS * TC;                             // twiddles
+  uint64_t* bar = reinterpret_cast<uint64_t*>(tws + P::L);         // [0] input, [1] spectrum
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bar + 2);
   const uint32_t bar_in = tc::smem_addr(bar), bar_g = tc::smem_addr(bar + 1);
   const uint32_t stg_a = tc::smem_addr(stg), gst_a = tc::smem_addr(gst);
   const float4* stg4 = reinterpret_cast<const float4*>(stg);
   const float4* gst4 = reinterpret_cast<const float4*>(gst);
   const int cp = threadIdx.x % NP;  // column pair 2cp, 2cp + 1 of the tile
-  const int t = threadIdx.x / NP;   // thread of the line (owns n2 = t in phases A, D)
-  // phases B, C: this thread's k1 and, split, its half h of the lane pair
-  int kb, h = 0;
-  if constexpr (SPLIT) decode<2, GP>(t, kb, h);
-  else kb = t;
+  const int t = threadIdx.x / NP;   // thread of the line
   const unsigned ntile = (unsigned)(a.ncols / TC);
-  const unsigned per_rhs = (unsigned)a.nplanes * ntile;
-  const int nact = a.active ? *a.n_active : a.nb;
-  const unsigned items = (unsigned)nact * per_rhs;  // < 2^31 (fwi_create caps the batch)
+  const unsigned grp = pair_group(ntile), ngrp = gridDim.x / grp;
+  const unsigned nact = (unsigned)(a.active ? *a.n_active : a.nb);
+  const unsigned items = ntile / grp * (unsigned)a.nplanes * nact;  // < 2^31 (fwi_create)
+  const unsigned per = (items + ngrp - 1) / ngrp;
+  const unsigned first = blockIdx.x / grp * per;
+  const unsigned last = blockIdx.x / grp >= ngrp ? first : min(first + per, items);
   const int box_rows = rows_in / nbox;
   const uint32_t tile_bytes = (uint32_t)(rows_in * TC * sizeof(float2));
-  const uint32_t g_bytes = (uint32_t)(G_ROWS * TC * sizeof(float2));
+  const uint32_t g_bytes = (uint32_t)(SM::G_ROWS * TC * sizeof(float2));
   const long long ls = a.line_stride;
   int dummy_err = 0;
   int* err = a.err ? a.err : &dummy_err;
+  auto has_n2 = [&](int i) { return C1 * TL == R2 || t + i * TL < R2; };
+  auto has_k1 = [&](int i) { return C3 * TL == R1 || t + i * TL < R1; };
 
-  auto rhs_of = [&](const ColItem& it) { return a.active ? a.active[it.slot] : it.slot; };
-  auto issue_input = [&](unsigned item) {
-    const ColItem it = col_item(item, (unsigned)nact, per_rhs, ntile, a.nplanes, true);
+  // item -> column tile, plane, right-hand side, frequency
+  struct Item { int tile, plane, rhs, l; };
+  auto item_of = [&](unsigned item) {
+    const unsigned q = item / nact, tg = q / (unsigned)a.nplanes;
+    Item it;
+    it.plane = (int)(q - tg * (unsigned)a.nplanes);
+    it.tile = (int)(tg * grp + blockIdx.x % grp);
+    const int slot = (int)(item - q * nact);
+    it.rhs = a.active ? a.active[slot] : slot;
+    it.l = a.freq_fixed >= 0 ? a.freq_fixed : (a.rhs0 + it.rhs) / a.n_elem;
+    return it;
+  };
+  auto issue_input = [&](const Item& it) {
     tc::mbar_arrive_expect_tx(bar_in, tile_bytes);
     for (int b = 0; b < nbox; ++b)
       tc::tma_load_3d(stg_a + (uint32_t)(b * box_rows * TC * sizeof(float2)), &map,
-                      2 * it.tile * TC, b * box_rows, rhs_of(it) * a.nplanes + it.plane, bar_in);
+                      2 * it.tile * TC, b * box_rows, it.rhs * a.nplanes + it.plane, bar_in);
   };
-  auto issue_spectrum = [&](unsigned item) {
-    const ColItem it = col_item(item, (unsigned)nact, per_rhs, ntile, a.nplanes, true);
-    const int l = a.freq_fixed >= 0 ? a.freq_fixed : (a.rhs0 + rhs_of(it)) / a.n_elem;
+  auto prefetch_input = [&](const Item& it) {
+    for (int b = 0; b < nbox; ++b)
+      tc::tma_prefetch_3d(&map, 2 * it.tile * TC, b * box_rows, it.rhs * a.nplanes + it.plane);
+  };
+  auto issue_spectrum = [&](const Item& it) {
     tc::mbar_arrive_expect_tx(bar_g, g_bytes);
-    tc::tma_load_3d(gst_a, &gmap, 2 * it.tile * TC, 0, l, bar_g);
+    for (int b = 0; b < SM::GBOX; ++b)
+      tc::tma_load_3d(gst_a + (uint32_t)(b * SM::G_BOX_ROWS * TC * sizeof(float2)), &gmap,
+                      2 * it.tile * TC, b * SM::G_BOX_ROWS, it.l, bar_g);
   };
 
   if (threadIdx.x == 0) {
@@ -367,114 +403,151 @@ col_pair_kernel(const ColArgs<float> a, const __grid_constant__ CUtensorMap map,
     *abort_flag = 0;
     tc::mbar_init_fence();
   }
-  for (int i = threadIdx.x; i < P::L; i += blockDim.x) {
-    const float2 w = a.tw[i];
-    twp[i] = make_float4(w.x, w.x, w.y, w.y);
-  }
+  for (int i = threadIdx.x; i < P::L; i += blockDim.x) tws[i] = a.tw[i];
   __syncthreads();
-  if (threadIdx.x == 0 && blockIdx.x < items) {
-    issue_input(blockIdx.x);
-    if (GS) issue_spectrum(blockIdx.x);
+  Item it = first < last ? item_of(first) : Item{0, 0, 0, 0}, nx = it;
+  if (threadIdx.x == 0 && first < last) {
+    issue_input(it);
+    issue_spectrum(it);
   }
   uint32_t par_in = 0, par_g = 0;
-  bool failed = false, bad = false;
-  for (unsigned item = blockIdx.x; item < items; item += gridDim.x) {
-    const ColItem it = col_item(item, (unsigned)nact, per_rhs, ntile, a.nplanes, true);
+  // new_g: the item has another spectrum tile than the one before it;
+  // g_copy (thread 0): a copy of one is in flight
+  bool failed = false, bad = false, new_g = true, g_copy = first < last;
+  for (unsigned item = first; item < last; ++item, it = nx) {
+    const bool more = item + 1 < last;
+    if (more) nx = item_of(item + 1);
     const int j = it.tile * TC + 2 * cp;
     const bool ok = tc::mbar_wait(bar_in, par_in, abort_flag, err, kColErrWait);
     PC v[P::E];
-    const u64 zero = pk(0.f, 0.f);
-    // phase-A samples x[R2 n1 + t] (n1 < R1/2; the rest is the zero padding)
+    // phase-A samples x[R2 n1 + n2], n1 < R1/2 (the rest is the zero padding)
 #pragma unroll
-    for (int n1 = 0; n1 < R1; ++n1)
-      v[n1] = (n1 < H1) ? from_interleaved(stg4[(R2 * n1 + t) * NP + cp]) : PC{zero, zero};
-    // every thread holds its samples (the input staging is free) and is done
-    // with the previous item's exchange; a failed wait (this item's input,
-    // or the previous item's spectrum) stops the CTA
+    for (int i = 0; i < C1; ++i)
+      if (has_n2(i))
+#pragma unroll
+        for (int n1 = 0; n1 < H1; ++n1)
+          v[i * R1 + n1] = from_interleaved(stg4[(R2 * n1 + t + i * TL) * NP + cp]);
+    // every thread holds its samples (the input staging is free: the next copy
+    // into it comes after the fence) and is done with the previous item's
+    // exchange; a failed wait (this item's input, or the previous item's
+    // spectrum) stops the CTA
+    if constexpr (!ALIAS) tc::fence_proxy_async();
     if (__syncthreads_or(!ok || bad)) {
       failed = true;
       break;
     }
     par_in ^= 1u;
-    const unsigned next = item + gridDim.x;
-    if (threadIdx.x == 0 && next < items) issue_input(next);
+    if (threadIdx.x == 0 && more) {
+      if constexpr (ALIAS) prefetch_input(nx);
+      else issue_input(nx);
+    }
     float2* __restrict__ out =
-        a.out + rhs_of(it) * a.out_rhs_stride + it.plane * a.out_plane_stride + j;
+        a.out + it.rhs * a.out_rhs_stride + it.plane * a.out_plane_stride + j;
 
-    // phase A: R1-point DFTs, twiddle w_L^{t k1}, y[t][k1] to the exchange
-    PDftHalfIn<R1, false>::run(v);
+    // phase A: R1-point DFTs, twiddle w_L^{n2 k1}, y[n2][k1] to the exchange
 #pragma unroll
-    for (int k1 = 0; k1 < R1; ++k1) {
-      PC z = v[k1];
-      if (k1 > 0 && t > 0) {
-        const float4 w = twp[t * k1];
-        z = ptw_tab(z, pk(w.x, w.y), pk(w.z, w.w));
+    for (int i = 0; i < C1; ++i) {
+      const int n2 = t + i * TL;
+      if (!has_n2(i)) continue;
+      PDftHalfIn<R1, false>::run(v + i * R1);
+#pragma unroll
+      for (int k1 = 0; k1 < R1; ++k1) {
+        PC z = v[i * R1 + k1];
+        if (k1 > 0 && n2 > 0) {
+          const float2 w = tws[n2 * k1];
+          z = ptw_tab(z, pk(w.x, w.x), pk(w.y, w.y));
+        }
+        sts_pc(ex + (n2 * R1P + k1) * NP + cp, z);
       }
-      sts_pc(ex + (t * R1 + k1) * NP + cp, z);
     }
-    // one thread waits for the staged spectrum; the barrier hands its
+    // one thread waits for a new spectrum tile; the barrier hands its
     // completion (and the copied data) to the others
-    if (GS && threadIdx.x == 0 && !tc::mbar_wait(bar_g, par_g, abort_flag, err, kColErrWait))
-      bad = true;
-    __syncthreads();
-    // phase B: R2-point DFTs over n2 (split: over the lane pair, n2 = 2m + h);
-    // v[kp] = X[kb + R1 k2] with k2 = kp (split: kp + Q2 h)
-#pragma unroll
-    for (int m = 0; m < NB; ++m) {
-      const int n2 = SPLIT ? 2 * m + h : m;
-      v[m] = lds_pc(ex + (n2 * R1 + kb) * NP + cp);
-    }
-    if constexpr (SPLIT) psplit_dft<NB, false>(v, h);
-    else PDft<R2, false>::run(v);
-    // product with the kernel spectrum (rows folded onto 0..L/2): the
-    // staged tile, or the columns (j, j + 1) of this item's frequency
-    const float4* __restrict__ gg = nullptr;
-    if constexpr (!GS) {
-      const int l = a.freq_fixed >= 0 ? a.freq_fixed : (a.rhs0 + rhs_of(it)) / a.n_elem;
-      gg = reinterpret_cast<const float4*>(a.ghat + (long long)l * a.ghat_freq_stride + j);
-    }
-#pragma unroll
-    for (int kp = 0; kp < NB; ++kp) {
-      const int row = spectrum_row<P>(kb, SPLIT ? kp + NB * h : kp, kp);
-      float4 g;
-      if constexpr (GS) g = gst4[row * NP + cp];
-      else g = __ldg(gg + (long long)row * (a.ncols / 2));
-      v[kp] = pmul(v[kp], pk(g.x, g.z), pk(g.y, g.w));
-    }
-    if constexpr (GS) {
-      __syncthreads();
-      // every thread is done with the staged spectrum: stage the next one
-      par_g ^= 1u;
-      if (threadIdx.x == 0 && next < items && !*abort_flag) issue_spectrum(next);
-    } else {
-      __syncthreads();  // every thread has read its phase-B values
-    }
-    // phase C: inverse DFTs over k2, twiddle w_L^{-n2 kb}, y[n2][kb]
-    if constexpr (SPLIT) psplit_idft<NB, true>(v, h);
-    else PDft<R2, true>::run(v);
-#pragma unroll
-    for (int m = 0; m < NB; ++m) {
-      const int n2 = SPLIT ? 2 * m + h : m;
-      PC z = v[m];
-      if (n2 > 0 && kb > 0) {
-        const float4 w = twp[n2 * kb];
-        z = ptw_tab_conj(z, pk(w.x, w.y), pk(w.z, w.w));
+    if (new_g && threadIdx.x == 0) {
+      if (tc::mbar_wait(bar_g, par_g, abort_flag, err, kColErrWait)) {
+        par_g ^= 1u;
+        g_copy = false;
+      } else {
+        bad = true;
       }
-      sts_pc(ex + (n2 * R1 + kb) * NP + cp, z);
+    }
+    __syncthreads();
+    // phase B: R2-point DFTs over n2, v[k2] = X[k1 + R1 k2]; product with the
+    // kernel spectrum (rows folded onto 0..L/2)
+#pragma unroll
+    for (int i = 0; i < C3; ++i) {
+      const int k1 = t + i * TL;
+      if (!has_k1(i)) continue;
+      PC* u = v + i * R2;
+#pragma unroll
+      for (int n2 = 0; n2 < R2; ++n2) u[n2] = lds_pc(ex + (n2 * R1P + k1) * NP + cp);
+      PDft<R2, false>::run(u);
+#pragma unroll
+      for (int k2 = 0; k2 < R2; ++k2) {
+        const int row = spectrum_row<P>(k1, k2, k2);
+        const float4 g = gst4[row * NP + cp];
+        u[k2] = pmul(u[k2], pk(g.x, g.z), pk(g.y, g.w));
+      }
+    }
+    // The exchange slots (n2, k1) of a k1 belong to its thread in phases B and
+    // C alike, so no barrier separates them; one before the next item's spectrum
+    // tile replaces this one.
+    new_g = more && (nx.tile != it.tile || nx.l != it.l);
+    if (new_g) {
+      tc::fence_proxy_async();
+      __syncthreads();
+      if (threadIdx.x == 0 && !bad) {
+        issue_spectrum(nx);
+        g_copy = true;
+      }
+    }
+    // phase C: inverse DFTs over k2, twiddle w_L^{-n2 k1}, y[n2][k1]
+#pragma unroll
+    for (int i = 0; i < C3; ++i) {
+      const int k1 = t + i * TL;
+      if (!has_k1(i)) continue;
+      PC* u = v + i * R2;
+      PDft<R2, true>::run(u);
+#pragma unroll
+      for (int n2 = 0; n2 < R2; ++n2) {
+        PC z = u[n2];
+        if (n2 > 0 && k1 > 0) {
+          const float2 w = tws[n2 * k1];
+          z = ptw_tab_conj(z, pk(w.x, w.x), pk(w.y, w.y));
+        }
+        sts_pc(ex + (n2 * R1P + k1) * NP + cp, z);
+      }
     }
     __syncthreads();
     // phase D: inverse R1-point DFTs of which the cropped half is formed
 #pragma unroll
-    for (int k1 = 0; k1 < R1; ++k1) v[k1] = lds_pc(ex + (t * R1 + k1) * NP + cp);
-    PDftHalfOut<R1, true>::run(v);
+    for (int i = 0; i < C1; ++i) {
+      const int n2 = t + i * TL;
+      if (!has_n2(i)) continue;
 #pragma unroll
-    for (int n1 = 0; n1 < H1; ++n1)
-      *reinterpret_cast<float4*>(out + (long long)(R2 * n1 + t) * ls) = to_interleaved(v[n1]);
+      for (int k1 = 0; k1 < R1; ++k1) v[i * R1 + k1] = lds_pc(ex + (n2 * R1P + k1) * NP + cp);
+    }
+    if constexpr (ALIAS) {
+      // the exchange is free: the next item's tile may land in it (the fence
+      // orders this thread's exchange accesses before the copy's writes)
+      tc::fence_proxy_async();
+      __syncthreads();
+      if (threadIdx.x == 0 && more) issue_input(nx);
+    }
+#pragma unroll
+    for (int i = 0; i < C1; ++i) {
+      const int n2 = t + i * TL;
+      if (!has_n2(i)) continue;
+      PC* u = v + i * R1;
+      PDftHalfOut<R1, true>::run(u);
+#pragma unroll
+      for (int n1 = 0; n1 < H1; ++n1)
+        *reinterpret_cast<float4*>(out + (long long)(R2 * n1 + n2) * ls) = to_interleaved(u[n1]);
+    }
   }
   // copies of a CTA that stopped early may still land in its shared memory
   if (failed && threadIdx.x == 0) {
     tc::mbar_wait_drain(bar_in, par_in, err, kColErrDrain);
-    if (GS) tc::mbar_wait_drain(bar_g, par_g, err, kColErrDrain);
+    if (g_copy) tc::mbar_wait_drain(bar_g, par_g, err, kColErrDrain);
   }
 }
 

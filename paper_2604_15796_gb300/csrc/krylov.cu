@@ -684,7 +684,7 @@ fwi_status apply_op_t(fwi_ctx* c, int kind, const void* m, int freq, int n_rhs,
 // context's full batch (scratch vectors) and keeps the fastest.  Variants
 // differ only in how many lines / columns a CTA holds; every one gives
 // bitwise-identical results.  Choices are cached in a text file keyed by
-// (architecture, precision, length, batch, pass).
+// (kernel generation, architecture, precision, length, batch, pass).
 std::string tune_cache_path() {
   const char* p = std::getenv("LIBFWI_TUNE_CACHE");
   if (p && *p) return p;
@@ -729,7 +729,7 @@ fwi_status autotune_t(fwi_ctx* c) {
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, c->device);
   cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, c->device);
   char base[160];
-  std::snprintf(base, sizeof(base), "sm%d%d|%s|d%d|%dx%dx%d|b%d|", major, minor,
+  std::snprintf(base, sizeof(base), "v2|sm%d%d|%s|d%d|%dx%dx%d|b%d|", major, minor,
                 sizeof(T) == 4 ? "c64" : "c128", c->dim, c->lx, c->ly, c->lz, c->batch);
   const std::string kb(base);
   const char* kinds[4] = {"row_fwd", "row_inv", "col_z", "col_y"};

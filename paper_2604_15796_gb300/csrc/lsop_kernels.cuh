@@ -547,6 +547,7 @@ row_fwd_kernel(const RowFwdArgs<T> a) {
     // shared memory of the previous item fully consumed (and, staged, this
     // item's rows are in registers: the staging area is free)
     if constexpr (STG) {
+      tc::fence_proxy_async();  // before the next copies into the staging area
       if (__syncthreads_or(!ok)) {
         failed = true;
         break;
@@ -966,6 +967,7 @@ __device__ __forceinline__ bool col_transform_store(const ColArgs<T>& a, int t, 
         }
       }
     }
+    if (gs) tc::fence_proxy_async();  // the next spectrum tile replaces this one
     __syncthreads();
     if (gs) hook.spectrum_done();
   }
@@ -1179,9 +1181,11 @@ col_tma_kernel(const ColArgs<float> a, const __grid_constant__ CUtensorMap map,
         }
       }
     }
-    // every thread holds its samples (the input staging is free) and is
-    // done with the previous item's exchange; a failed wait (this item's
-    // input, or the previous item's spectrum) stops the CTA
+    // every thread holds its samples (the input staging is free: the next
+    // copy into it comes after the fence) and is done with the previous item's
+    // exchange; a failed wait (this item's input, or the previous item's
+    // spectrum) stops the CTA
+    tc::fence_proxy_async();
     if (__syncthreads_or(!ok || bad)) {
       failed = true;
       break;
@@ -1366,19 +1370,17 @@ cudaError_t launch_row_inv(const RowInvArgs<T>& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Tensor map of the kernel spectrum for the convolution's staging: rows
-// 0..L/2 of TC columns of one frequency per box.  False when the box does
-// not fit (L/2 + 1 > 256 rows) or the staging would cost occupancy.
+// Tensor map of the kernel spectrum for the convolution's staging: boxes of
+// box_rows (at most 256) rows of TC columns of one frequency.
 template <int L, int TC>
-bool col_spectrum_map(const ColArgs<float>& a, int rows_in, CUtensorMap* map) {
+bool col_spectrum_map(const ColArgs<float>& a, int box_rows, CUtensorMap* map) {
   if (!a.gstage || a.mode != C_CONV || !a.ghat || a.n_freq < 1) return false;
-  if (L / 2 + 1 > 256 || ColTmaSmem<L, TC>::bytes(rows_in, true) > 76 * 1024) return false;
   tc::TensorMapEncodeFn enc = tc::tensor_map_encoder();
   if (!enc || ((uintptr_t)a.ghat & 15) || (a.ncols * 8) % 16 || (a.ghat_freq_stride * 8) % 16)
     return false;
   const cuuint64_t dims[3] = {(cuuint64_t)2 * a.ncols, (cuuint64_t)L, (cuuint64_t)a.n_freq};
   const cuuint64_t strides[2] = {(cuuint64_t)a.ncols * 8, (cuuint64_t)a.ghat_freq_stride * 8};
-  const cuuint32_t box[3] = {(cuuint32_t)(2 * TC), (cuuint32_t)(L / 2 + 1), 1};
+  const cuuint32_t box[3] = {(cuuint32_t)(2 * TC), (cuuint32_t)box_rows, 1};
   const cuuint32_t estr[3] = {1, 1, 1};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float2*>(a.ghat), dims, strides,
              box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -1414,7 +1416,8 @@ bool col_tensor_map(const ColArgs<float>& a, CUtensorMap* map, int* rows_in, int
   return true;
 }
 
-// The two-column convolution stores 16-byte column pairs.
+// The two-column convolution stores 16-byte column pairs, and takes its
+// spectrum from a staged tile.
 template <typename T> bool col_pair_ok(const ColArgs<T>& a) {
   return a.mode == C_CONV && a.pairs && a.ghat && ((uintptr_t)a.out & 15) == 0 &&
          a.out_rhs_stride % 2 == 0 && a.line_stride % 2 == 0 &&
@@ -1430,19 +1433,22 @@ cudaError_t launch_col(const ColArgs<T>& a, cudaStream_t s) {
     int rows_in = 0, nbox = 0;
     if (col_tensor_map<L, tc>(a, &map, &rows_in, &nbox)) {
       using SM = ColTmaSmem<L, tc>;
+      if constexpr (tc % 2 == 0) {
+        using PP = typename PairPlanFor<L>::type;
+        using PSM = ColPairSmem<PP, tc>;
+        if (col_pair_ok(a) && col_spectrum_map<L, tc>(a, PSM::G_BOX_ROWS, &gmap)) {
+          auto k = col_pair_kernel<PP, tc>;
+          const size_t smem = PSM::bytes(rows_in);
+          GridCache& gc = gcache<L, T, 6, VAR>();
+          cudaError_t e = grid_for(k, tc / 2 * PP::TL, smem, gc);
+          if (e != cudaSuccess) return e;
+          k<<<gc.blocks.load(), tc / 2 * PP::TL, smem, s>>>(a, map, gmap, rows_in, nbox);
+          return cudaGetLastError();
+        }
+      }
       if constexpr (L / 2 + 1 <= 256) {
-        if (col_spectrum_map<L, tc>(a, rows_in, &gmap)) {
-          if constexpr (pair_plan<P>() && tc % 2 == 0) {
-            if (col_pair_ok(a)) {
-              auto k = col_pair_kernel<P, tc, true>;
-              const size_t smem = ColPairSmem<L, tc>::bytes(rows_in, true);
-              GridCache& gc = gcache<L, T, 6, VAR>();
-              cudaError_t e = grid_for(k, tc / 2 * P::TL, smem, gc);
-              if (e != cudaSuccess) return e;
-              k<<<gc.blocks.load(), tc / 2 * P::TL, smem, s>>>(a, map, gmap, rows_in, nbox);
-              return cudaGetLastError();
-            }
-          }
+        if (SM::bytes(rows_in, true) <= 76 * 1024 &&
+            col_spectrum_map<L, tc>(a, SM::G_ROWS, &gmap)) {
           auto k = col_tma_kernel<P, tc, true>;
           const size_t smem = SM::bytes(rows_in, true);
           GridCache& gc = gcache<L, T, 5, VAR>();
@@ -1461,19 +1467,6 @@ cudaError_t launch_col(const ColArgs<T>& a, cudaStream_t s) {
       {
         cudaError_t e = grid_for(kp, tc * P::TL, col_smem_v<L, T, VAR>(), gcp);
         if (e != cudaSuccess) return e;
-      }
-      if constexpr (pair_plan<P>() && tc % 2 == 0) {
-        // the spectrum from global memory (16-byte column pairs)
-        if (col_pair_ok(a) && ((uintptr_t)a.ghat & 15) == 0 && a.ncols % 2 == 0 &&
-            a.ghat_freq_stride % 2 == 0) {
-          auto k = col_pair_kernel<P, tc, false>;
-          const size_t smem = ColPairSmem<L, tc>::bytes(rows_in, false);
-          GridCache& gc = gcache<L, T, 7, VAR>();
-          cudaError_t e = grid_for(k, tc / 2 * P::TL, smem, gc);
-          if (e != cudaSuccess) return e;
-          k<<<gc.blocks.load(), tc / 2 * P::TL, smem, s>>>(a, map, gmap, rows_in, nbox);
-          return cudaGetLastError();
-        }
       }
       auto k = col_tma_kernel<P, tc, false>;
       const size_t smem = SM::bytes(rows_in, false);

@@ -83,8 +83,11 @@ __device__ __forceinline__ void fence_before_sync() {
 __device__ __forceinline__ void fence_after_sync() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
-// Make this thread's generic-proxy shared-memory writes visible to the
-// tensor core (async proxy).
+// Order this thread's shared-memory accesses before later ones of the async
+// proxy: writes, so that the tensor core sees them, and reads, before a barrier
+// after which another thread lets a TMA or bulk copy overwrite what was read.
+// (A barrier alone does not wait for loads still in flight: with another
+// kernel's CTAs on the SM, copies were seen to land before them.)
 __device__ __forceinline__ void fence_proxy_async() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
@@ -217,6 +220,13 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
+// L2 prefetch of one box (nothing to wait for).
+__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int x, int y, int z) {
+  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(
+                   reinterpret_cast<uint64_t>(map)),
+               "r"(x), "r"(y), "r"(z)
+               : "memory");
+}
 
 // 16-byte global -> shared copy; src_bytes 0 fills zeros.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
