@@ -49,6 +49,7 @@ __device__ inline void tile_of(int ty, int nbe, int sym, int& eb, int& jb) {
   eb = ty - jb * (jb + 1) / 2;
 }
 
+// FP32 fields on CUDA cores.
 template <typename T>
 __global__ void __launch_bounds__(256)
 contract_kernel(const cplx<T>* __restrict__ X, const cplx<T>* __restrict__ a,
@@ -120,29 +121,163 @@ contract_kernel(const cplx<T>* __restrict__ X, const cplx<T>* __restrict__ a,
     }
 }
 
+// ---- FP64 fields ----------------------------------------------------------
+// FP64 issues at about two multiply-adds per clock and SM on this part, so the
+// FP64 products are bound by that alone, whatever the tile: one complex output
+// per thread (16 x 16 tiles) wastes the least on padding, computes the smallest
+// triangle of a symmetric product, and splits into enough CTAs for the chip.
+// 64^2 pixels x 32 elements on one GB300, with the 64 x 64 tiles before and now:
+// contraction 225 -> 49 us, J^H 230 -> 63 us a launch (floor 27 us).
+constexpr int TD = 16;
+
+__global__ void __launch_bounds__(TD * TD)
+contract_f64_kernel(const double2* __restrict__ X, const double2* __restrict__ a,
+                    const double2* __restrict__ Q, double2* __restrict__ part, int NE,
+                    long long N, int n_freq, long long chunk, int sym) {
+  __shared__ double2 Xs[KC][TD + 1];
+  __shared__ double2 Qs[KC][TD + 1];
+  static_assert(KC == TD, "one load per thread and chunk");
+  const int s = blockIdx.y, l = blockIdx.z;
+  int eb, jb;
+  tile_of(blockIdx.x, (NE + TD - 1) / TD, sym, eb, jb);
+  const int c = threadIdx.x % TD, r = threadIdx.x / TD;
+  const long long n_begin = (long long)s * chunk;
+  const long long n_end = (n_begin + chunk < N) ? n_begin + chunk : N;
+  const int e = eb * TD + r, j = jb * TD + r;  // rows this thread loads
+  const double2* Xe = X + ((long long)l * NE + e) * N;
+  const double2* Qj = Q + ((long long)l * NE + j) * N;
+  const double2 zero = make_double2(0.0, 0.0);
+  double2 acc = zero;
+  for (long long n0 = n_begin; n0 < n_end; n0 += KC) {
+    const long long n = n0 + c;
+    double2 xv = zero, qv = zero;
+    if (n < n_end) {
+      if (e < NE) {
+        xv = Xe[n];
+        if (a) xv = cmul(xv, a[n]);
+      }
+      if (j < NE) qv = Qj[n];
+    }
+    Xs[c][r] = xv;
+    Qs[c][r] = qv;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < KC; ++k) {
+      const double2 x = Xs[k][r], q = Qs[k][c];  // output (eb TD + r, jb TD + c)
+      acc.x += x.x * q.x - x.y * q.y;
+      acc.y += x.x * q.y + x.y * q.x;
+    }
+    __syncthreads();
+  }
+  const int jo = jb * TD + c;
+  if (e < NE && jo < NE) part[(((long long)s * n_freq + l) * NE + e) * NE + jo] = acc;
+}
+
+// The mix over rows e of one 64-row block (as many z partials as the 64 x 64
+// tiles had), 16 rows at a time.
+template <bool FUSED>
+__global__ void __launch_bounds__(TD * TD)
+mix_f64_kernel(const double2* __restrict__ B, const double2* __restrict__ Q, int conjQ,
+               const double2* __restrict__ X, double2* __restrict__ out,
+               const double* __restrict__ scale, int NE, long long N) {
+  __shared__ double2 Bs[KC][TD + 1];
+  __shared__ double2 Qs[KC][TD + 1];
+  const int l = blockIdx.z, nbe = gridDim.y, e_end = min((int)(blockIdx.y + 1) * TB, NE);
+  const int c = threadIdx.x % TD, r = threadIdx.x / TD;
+  const long long n = (long long)blockIdx.x * TD + c;
+  const double2* Bl = B + (long long)l * NE * NE;
+  const double2* Ql = Q + (long long)l * NE * N;
+  const double2 zero = make_double2(0.0, 0.0);
+  const double f = scale[l];
+  double2 z = zero;
+  for (int e0 = blockIdx.y * TB; e0 < e_end; e0 += TD) {
+    const int e = e0 + r;
+    double2 acc = zero;
+    for (int j0 = 0; j0 < NE; j0 += KC) {
+      Bs[c][r] = (e < NE && j0 + c < NE) ? Bl[(long long)e * NE + j0 + c] : zero;
+      double2 q = (j0 + r < NE && n < N) ? Ql[(long long)(j0 + r) * N + n] : zero;
+      if (conjQ) q.y = -q.y;
+      Qs[r][c] = q;
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < KC; ++k) {
+        const double2 b = Bs[k][r], v = Qs[k][c];
+        acc.x += b.x * v.x - b.y * v.y;
+        acc.y += b.x * v.y + b.y * v.x;
+      }
+      __syncthreads();
+    }
+    if (e < NE && n < N) {
+      const long long i = ((long long)l * NE + e) * N + n;
+      if (FUSED) z = cadd(z, cmulc(acc, X[i]));  // W * conj(X)
+      else out[i] = make_double2(acc.x * f, acc.y * f);
+    }
+  }
+  if (!FUSED) return;
+  Bs[r][c] = z;
+  __syncthreads();
+  if (r == 0 && n < N) {
+    double2 t = zero;
+#pragma unroll
+    for (int k = 0; k < TD; ++k) t = cadd(t, Bs[k][c]);
+    out[((long long)l * nbe + blockIdx.y) * N + n] = make_double2(t.x * f, t.y * f);
+  }
+}
+
 // Y[l][e][j] = scale_l * sum_s part[s][l][e][j]  (FP64, fixed order); with
 // sym, entries below the computed tiles (eb > jb) are read transposed.
-template <typename T>
+// LANES (a power of two up to 32) neighbouring threads share one output, each
+// adding every LANES-th partial: 8 where there are few outputs and many splits,
+// whose loads would otherwise form one serial chain per output.
+template <typename T, int LANES>
 __global__ void contract_reduce_kernel(double2* Y, const cplx<T>* part, int split,
                                        long long per_split, int NE2, const double* scale,
-                                       int NE, int sym) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < per_split;
-       i += (long long)gridDim.x * blockDim.x) {
-    long long src = i;
-    if (sym) {
-      const long long l = i / NE2;
-      const int e = (int)((i % NE2) / NE), j = (int)(i % NE);
-      if (e / TB > j / TB) src = l * NE2 + (long long)j * NE + e;
-    }
+                                       int NE, int sym_tile) {
+  const int lane = threadIdx.x % LANES;
+  const long long n = (per_split * LANES + 31) / 32 * 32;  // whole warps
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
+       t += (long long)gridDim.x * blockDim.x) {
+    const long long i = t / LANES;
     double sx = 0.0, sy = 0.0;
-    for (int s = 0; s < split; ++s) {
-      const cplx<T> v = part[(long long)s * per_split + src];
-      sx += (double)v.x;
-      sy += (double)v.y;
+    if (i < per_split) {
+      long long src = i;
+      if (sym_tile) {
+        const long long l = i / NE2;
+        const int e = (int)((i % NE2) / NE), j = (int)(i % NE);
+        if (e / sym_tile > j / sym_tile) src = l * NE2 + (long long)j * NE + e;
+      }
+#pragma unroll 4
+      for (int s = lane; s < split; s += LANES) {
+        const cplx<T> v = part[(long long)s * per_split + src];
+        sx += (double)v.x;
+        sy += (double)v.y;
+      }
     }
-    const double f = scale[i / NE2];
-    Y[i] = make_double2(sx * f, sy * f);
+#pragma unroll
+    for (int off = LANES / 2; off > 0; off >>= 1) {
+      sx += __shfl_down_sync(0xffffffffu, sx, off, LANES);
+      sy += __shfl_down_sync(0xffffffffu, sy, off, LANES);
+    }
+    if (lane == 0 && i < per_split) {
+      const double f = scale[i / NE2];
+      Y[i] = make_double2(sx * f, sy * f);
+    }
   }
+}
+
+// Reduction of the split partials; sym_tile: the tile edge when only tiles on
+// and above the diagonal were computed, else 0.
+template <typename T>
+cudaError_t contract_reduce(fwi_ctx* c, double2* Y, int split, long long per, int sym_tile) {
+  const int ne = c->n_elem;
+  const cplx<T>* part = (const cplx<T>*)c->jsplit;
+  if (per < 16384 && split >= 16)
+    contract_reduce_kernel<T, 8><<<blocks_for(per * 8, 256, c->n_sm * 8), 256, 0, c->stream>>>(
+        Y, part, split, per, ne * ne, c->red, ne, sym_tile);
+  else
+    contract_reduce_kernel<T, 1><<<blocks_for(per, 256, c->n_sm * 8), 256, 0, c->stream>>>(
+        Y, part, split, per, ne * ne, c->red, ne, sym_tile);
+  return cudaGetLastError();
 }
 
 template <typename T, bool FUSED>
@@ -345,10 +480,10 @@ template <typename T> struct Jac {
     return s;
   }
 
-  static int split_for(fwi_ctx* c) {
-    const int nbe = (c->n_elem + TB - 1) / TB;
-    const int tiles = nbe * nbe * c->n_freq;
-    int split = (c->n_sm * 6 + tiles - 1) / tiles;
+  // FP64: two CTAs per SM keep its FP64 units busy
+  static constexpr int TILE = sizeof(T) == 8 ? TD : TB;
+  static int split_for(fwi_ctx* c, int tiles) {
+    int split = (c->n_sm * (sizeof(T) == 8 ? 2 : 6) + tiles - 1) / tiles;
     const long long max_split = (c->N + KC - 1) / KC;
     if (split > max_split) split = (int)max_split;
     if (split < 1) split = 1;
@@ -369,34 +504,31 @@ template <typename T> struct Jac {
         const int split = tc_contract_partials(c, X, a, Q, (float2*)c->jsplit);
         if (split < 0) return FWI_ERR_CUDA;
         Prof p(c, KC_MISC);
-        contract_reduce_kernel<T><<<blocks_for(per, 256, c->n_sm * 8), 256, 0, c->stream>>>(
-            Y, (const cplx<T>*)c->jsplit, split, per, c->n_elem * c->n_elem, c->red, c->n_elem,
-            0);
-        FWI_CUDA(c, cudaGetLastError());
+        FWI_CUDA(c, contract_reduce<T>(c, Y, split, per, 0));
         return FWI_OK;
       }
     }
-    const int nbe = (c->n_elem + TB - 1) / TB;
-    const int split = split_for(c);
+    const int nbe = (c->n_elem + TILE - 1) / TILE;
     const int sym = (X == Q) ? 1 : 0;
+    const int tiles = sym ? nbe * (nbe + 1) / 2 : nbe * nbe;
+    const int split = split_for(c, (sizeof(T) == 8 ? tiles : nbe * nbe) * c->n_freq);
     long long chunk = (c->N + split - 1) / split;
     chunk = ((chunk + KC - 1) / KC) * KC;
-    dim3 grid(split, sym ? nbe * (nbe + 1) / 2 : nbe * nbe, c->n_freq);
+    dim3 grid(split, tiles, c->n_freq);
     const double fe = (double)c->n_freq * c->n_elem * c->N;
     {
       Prof p(c, KC_CONTRACT, (2.0 * fe + (a ? c->N : 0)) * sizeof(cplx<T>),
              8.0 * fe * c->n_elem);
-      contract_kernel<T><<<grid, 256, 0, c->stream>>>(X, a, Q, (cplx<T>*)c->jsplit, c->n_elem,
-                                                      c->N, c->n_freq, chunk, sym);
+      if constexpr (std::is_same<T, double>::value)
+        contract_f64_kernel<<<dim3(tiles, split, c->n_freq), TD * TD, 0, c->stream>>>(
+            X, a, Q, (double2*)c->jsplit, c->n_elem, c->N, c->n_freq, chunk, sym);
+      else
+        contract_kernel<T><<<grid, 256, 0, c->stream>>>(X, a, Q, (cplx<T>*)c->jsplit, c->n_elem,
+                                                        c->N, c->n_freq, chunk, sym);
     }
     FWI_CUDA(c, cudaGetLastError());
-    {
-      Prof p(c, KC_MISC);
-      contract_reduce_kernel<T><<<blocks_for(per, 256, c->n_sm * 8), 256, 0, c->stream>>>(
-          Y, (const cplx<T>*)c->jsplit, split, per, c->n_elem * c->n_elem, c->red, c->n_elem,
-          sym);
-    }
-    FWI_CUDA(c, cudaGetLastError());
+    Prof p(c, KC_MISC);
+    FWI_CUDA(c, contract_reduce<T>(c, Y, split, per, sym ? TILE : 0));
     return FWI_OK;
   }
 
@@ -584,9 +716,16 @@ template <typename T> static fwi_status adjoint_sources_t(fwi_ctx* c, void* out)
   dim3 grid((unsigned)((c->N + TB - 1) / TB), (c->n_elem + TB - 1) / TB, c->n_freq);
   const double fe = (double)c->n_freq * c->n_elem * c->N;
   Prof p(c, KC_MIX_SOURCES, 2.0 * fe * sizeof(cplx<T>), 8.0 * fe * c->n_elem);
-  mix_kernel<T, false><<<grid, 256, 0, c->stream>>>(
-      (const cplx<T>*)c->dF, (const cplx<T>*)c->p0, 0, nullptr, (cplx<T>*)out, c->red,
-      c->n_elem, c->N);
+  if constexpr (std::is_same<T, double>::value) {
+    grid.x = (unsigned)((c->N + TD - 1) / TD);
+    mix_f64_kernel<false><<<grid, TD * TD, 0, c->stream>>>(
+        (const double2*)c->dF, (const double2*)c->p0, 0, nullptr, (double2*)out, c->red,
+        c->n_elem, c->N);
+  } else {
+    mix_kernel<T, false><<<grid, 256, 0, c->stream>>>(
+        (const cplx<T>*)c->dF, (const cplx<T>*)c->p0, 0, nullptr, (cplx<T>*)out, c->red,
+        c->n_elem, c->N);
+  }
   FWI_CUDA(c, cudaGetLastError());
   return FWI_OK;
 }
@@ -683,9 +822,16 @@ template <typename T> static fwi_status jac_adjoint_t(fwi_ctx* c, const double2*
   {
     const double fe = (double)c->n_freq * c->n_elem * c->N;
     Prof p(c, KC_MIX_JH, 2.0 * fe * sizeof(cplx<T>), 8.0 * fe * c->n_elem + 8.0 * fe);
-    mix_kernel<T, true><<<grid, 256, 0, c->stream>>>(
-        (const cplx<T>*)c->dF, (const cplx<T>*)receiver_fields(c), 1,
-        (const cplx<T>*)c->fields, (cplx<T>*)c->zpart, c->red, c->n_elem, c->N);
+    if constexpr (std::is_same<T, double>::value) {
+      grid.x = (unsigned)((c->N + TD - 1) / TD);
+      mix_f64_kernel<true><<<grid, TD * TD, 0, c->stream>>>(
+          (const double2*)c->dF, (const double2*)receiver_fields(c), 1,
+          (const double2*)c->fields, (double2*)c->zpart, c->red, c->n_elem, c->N);
+    } else {
+      mix_kernel<T, true><<<grid, 256, 0, c->stream>>>(
+          (const cplx<T>*)c->dF, (const cplx<T>*)receiver_fields(c), 1,
+          (const cplx<T>*)c->fields, (cplx<T>*)c->zpart, c->red, c->n_elem, c->N);
+    }
   }
   FWI_CUDA(c, cudaGetLastError());
   Prof p(c, KC_MISC);
