@@ -457,10 +457,14 @@ typedef struct fwi_tuning {
                            one chain.  Results are bitwise the same. */
   int debug_stall_once; /* test of the failure path: 1 makes the next
                            tensor-core contraction withhold its first
-                           pipeline stage, so that its bounded waits give up
-                           after about 1 s and the call returns FWI_ERR_CUDA
-                           ("pipeline wait timed out"); the context stays
-                           usable.  Applies once; reads back as 0. */
+                           pipeline stage, or the next single operator
+                           application wait for more spectrum bytes than its
+                           convolution copies, whichever comes first, so that
+                           its bounded waits give up after about 1 s and the
+                           call (or, after one that does not synchronise, the
+                           next that does) returns FWI_ERR_CUDA ("pipeline
+                           wait timed out"); the context stays usable.
+                           Applies once; reads back as 0. */
   int col_tma;          /* 1 (default): the FP32 column passes stage their
                            input tiles (and, for the 3-D and smaller 2-D
                            convolutions, their kernel-spectrum tiles) in

@@ -389,8 +389,10 @@ col_pair_kernel(const ColArgs<float> a, const __grid_constant__ CUtensorMap map,
     for (int b = 0; b < nbox; ++b)
       tc::tma_prefetch_3d(&map, 2 * it.tile * TC, b * box_rows, it.rhs * a.nplanes + it.plane);
   };
+  uint32_t g_armed = 0;  // spectrum copies issued (thread 0)
   auto issue_spectrum = [&](const Item& it) {
-    tc::mbar_arrive_expect_tx(bar_g, g_bytes);
+    ++g_armed;
+    tc::mbar_arrive_expect_tx(bar_g, g_bytes + (a.stall ? 16u : 0u));
     for (int b = 0; b < SM::GBOX; ++b)
       tc::tma_load_3d(gst_a + (uint32_t)(b * SM::G_BOX_ROWS * TC * sizeof(float2)), &gmap,
                       2 * it.tile * TC, b * SM::G_BOX_ROWS, it.l, bar_g);
@@ -411,9 +413,8 @@ col_pair_kernel(const ColArgs<float> a, const __grid_constant__ CUtensorMap map,
     issue_spectrum(it);
   }
   uint32_t par_in = 0, par_g = 0;
-  // new_g: the item has another spectrum tile than the one before it;
-  // g_copy (thread 0): a copy of one is in flight
-  bool failed = false, bad = false, new_g = true, g_copy = first < last;
+  // new_g: the item has another spectrum tile than the one before it
+  bool failed = false, bad = false, new_g = true;
   for (unsigned item = first; item < last; ++item, it = nx) {
     const bool more = item + 1 < last;
     if (more) nx = item_of(item + 1);
@@ -463,12 +464,8 @@ col_pair_kernel(const ColArgs<float> a, const __grid_constant__ CUtensorMap map,
     // one thread waits for a new spectrum tile; the barrier hands its
     // completion (and the copied data) to the others
     if (new_g && threadIdx.x == 0) {
-      if (tc::mbar_wait(bar_g, par_g, abort_flag, err, kColErrWait)) {
-        par_g ^= 1u;
-        g_copy = false;
-      } else {
-        bad = true;
-      }
+      if (tc::mbar_wait(bar_g, par_g, abort_flag, err, kColErrWait)) par_g ^= 1u;
+      else bad = true;
     }
     __syncthreads();
     // phase B: R2-point DFTs over n2, v[k2] = X[k1 + R1 k2]; product with the
@@ -495,10 +492,7 @@ col_pair_kernel(const ColArgs<float> a, const __grid_constant__ CUtensorMap map,
     if (new_g) {
       tc::fence_proxy_async();
       __syncthreads();
-      if (threadIdx.x == 0 && !bad) {
-        issue_spectrum(nx);
-        g_copy = true;
-      }
+      if (threadIdx.x == 0 && !bad) issue_spectrum(nx);
     }
     // phase C: inverse DFTs over k2, twiddle w_L^{-n2 k1}, y[n2][k1]
 #pragma unroll
@@ -544,10 +538,12 @@ col_pair_kernel(const ColArgs<float> a, const __grid_constant__ CUtensorMap map,
         *reinterpret_cast<float4*>(out + (long long)(R2 * n1 + n2) * ls) = to_interleaved(u[n1]);
     }
   }
-  // copies of a CTA that stopped early may still land in its shared memory
-  if (failed && threadIdx.x == 0) {
-    tc::mbar_wait_drain(bar_in, par_in, err, kColErrDrain);
-    if (g_copy) tc::mbar_wait_drain(bar_g, par_g, err, kColErrDrain);
+  // copies of a CTA that stopped early may still land in its shared memory: the
+  // input of the item it stopped at, and the spectrum whose wait gave up, be it
+  // the last item's (which no later item's `failed` follows)
+  if (threadIdx.x == 0) {
+    if (failed) tc::mbar_wait_drain(bar_in, par_in, err, kColErrDrain);
+    tc::mbar_drain_armed(bar_g, g_armed, err, kColErrDrain);
   }
 }
 

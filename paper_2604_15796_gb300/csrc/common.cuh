@@ -93,6 +93,7 @@ template <typename T> struct ColArgs {
   int tma;                  // FP32, zero-padded input: stage tiles with TMA
   int gstage;               // with tma: also stage the kernel-spectrum tiles
   int pairs;                // with gstage: two columns per thread where the plan allows
+  int stall;                // test of the failure path: spectrum copies announce too many bytes
   int* err;                 // error word of bounded waits (or NULL)
 };
 

@@ -90,7 +90,7 @@ struct fwi_ctx {
   int jac_tma = 1;                  // tensor-core contractions take raw tiles by TMA
   int row_stage = 1;                // forward row pass stages its rows (FP32)
   int col_pairs = 1;                // convolution: two columns per thread (FP32)
-  int tc_stall = 0;                 // next contraction withholds its first stage (test)
+  int tc_stall = 0;                 // next staged call stalls once (test: debug_stall_once)
   double* red = nullptr;            // reduction scratch (doubles)
   double* h_red = nullptr;          // pinned host mirror
   int red_n = 0;

@@ -662,6 +662,8 @@ fwi_status apply_op_t(fwi_ctx* c, int kind, const void* m, int freq, int n_rhs,
   }
   Batch<T> b = make_batch<T>(c, (cplx<T>*)c->kv[0], 0, n_rhs);
   b.cz.freq_fixed = freq;  // every vector of the call is at frequency `freq`
+  b.cz.stall = c->tc_stall;
+  c->tc_stall = 0;  // one launch
   const cplx<T>* src = (const cplx<T>*)in;
   if (kind == 0) {  // K
     FWI_CUDA(c, row_fwd(b, RF_PLAIN, false, n_rhs, src, 0, 0));

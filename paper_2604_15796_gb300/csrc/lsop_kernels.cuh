@@ -1110,10 +1110,12 @@ col_tma_kernel(const ColArgs<float> a, const __grid_constant__ CUtensorMap map,
       tc::tma_load_3d(stg_a + (uint32_t)(b * box_rows * TC * sizeof(V)), &map, 2 * it.tile * TC,
                   b * box_rows, rhs_of(it) * a.nplanes + it.plane, bar_in);
   };
+  uint32_t g_armed = 0;  // spectrum copies issued (thread 0)
   auto issue_spectrum = [&](unsigned item) {
     const ColItem it = col_item(item, (unsigned)nact, per_rhs, ntile, a.nplanes, slot_fast);
     const int l = a.freq_fixed >= 0 ? a.freq_fixed : (a.rhs0 + rhs_of(it)) / a.n_elem;
-    tc::mbar_arrive_expect_tx(bar_g, g_bytes);
+    ++g_armed;
+    tc::mbar_arrive_expect_tx(bar_g, g_bytes + (a.stall ? 16u : 0u));
     tc::tma_load_3d(gst_a, &gmap, 2 * it.tile * TC, 0, l, bar_g);
   };
 
@@ -1196,10 +1198,12 @@ col_tma_kernel(const ColArgs<float> a, const __grid_constant__ CUtensorMap map,
       col_transform_store<P, float, TC, true>(a, t, smc, v, rhs, j, out, tws);
     }
   }
-  // copies of a CTA that stopped early may still land in its shared memory
-  if (failed && threadIdx.x == 0) {
-    tc::mbar_wait_drain(bar_in, par_in, err, kColErrDrain);
-    if (use_g) tc::mbar_wait_drain(bar_g, par_g, err, kColErrDrain);
+  // copies of a CTA that stopped early may still land in its shared memory: the
+  // input of the item it stopped at, and the spectrum whose wait gave up, be it
+  // the last item's (which no later item's `failed` follows; par_g has moved on)
+  if (threadIdx.x == 0) {
+    if (failed) tc::mbar_wait_drain(bar_in, par_in, err, kColErrDrain);
+    tc::mbar_drain_armed(bar_g, g_armed, err, kColErrDrain);
   }
 }
 

@@ -187,6 +187,16 @@ __device__ __forceinline__ void mbar_wait_drain(uint32_t bar, uint32_t parity, i
   }
 }
 
+// The same for a barrier that copies complete on, of which one thread armed
+// `armed` phases, each after the one before had completed: a CTA that gives up
+// waits for the phase still open, if there is one, before it exits, so that no
+// copy lands in shared memory that is no longer its own.  Returns at once when
+// every armed phase has completed.
+__device__ __forceinline__ void mbar_drain_armed(uint32_t bar, uint32_t armed, int* err,
+                                                 int code) {
+  if (armed) mbar_wait_drain(bar, (armed - 1) & 1u, err, code);
+}
+
 // ---- copies ----
 // cuTensorMapEncodeTiled, taken from the driver through the runtime (the
 // library does not link libcuda); NULL if the driver does not offer it.

@@ -613,9 +613,10 @@ class Context:
         self._check(fwi_set_tuning(self.handle, byref(t)))
 
     def debug_stall_once(self):
-        """Test of the failure path: the next tensor-core contraction
-        withholds its first pipeline stage, so that its bounded waits give up
-        (about 1 s) and the call raises FwiError (FWI_ERR_CUDA)."""
+        """Test of the failure path: the next tensor-core contraction or
+        single operator application stalls, so that its bounded waits give up
+        (about 1 s) and the call, or the next one that synchronises, raises
+        FwiError (FWI_ERR_CUDA)."""
         t = fwi_tuning()
         self._check(fwi_get_tuning(self.handle, byref(t)))
         t.debug_stall_once = 1

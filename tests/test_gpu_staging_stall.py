@@ -1,0 +1,41 @@
+"""A convolution whose staged spectrum never completes (debug_stall_once: the copy's
+barrier expects 16 bytes more than arrive) gives up its bounded wait, waits, again
+bounded, for the copy it has in flight, reports the error and leaves the context
+usable.  Both limits are 1 s, so a CTA that left without the second wait, its
+copy still in flight, would return in half the time: checked where the wait that
+gives up is the CTA's last (one item) and where other items follow."""
+import time
+
+import numpy as np
+import pytest
+
+from gpu_common import contrast, small_workload, to_gpu, to_np
+from paper_2604_15796_gb300 import phantoms
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n_rhs", [3, 600])
+@pytest.mark.parametrize("pairs", [True, False])
+def test_stalled_spectrum_copy_is_waited_for(pairs, n_rhs):
+    import torch
+    from paper_2604_15796_gb300 import build, libfwi
+    build.build()
+    w = small_workload((64, 32), n_elem=100, pitch=0.03e-3, freqs=np.linspace(1e6, 3e6, 6))
+    ctx = libfwi.Context(w.shape, w.h, w.c0, w.elem, w.freqs)
+    ctx.set_col_pairs(pairs)
+    m = to_gpu(contrast(w), torch.complex128)
+    v = to_gpu(phantoms.complex_normal((n_rhs,) + tuple(w.shape), 3), torch.complex64)
+    ref = to_np(ctx.apply("A", v, 1, m))
+    ctx.debug_stall_once()
+    t0 = time.perf_counter()
+    to_np(ctx.apply("A", v, 1, m))
+    waited = time.perf_counter() - t0
+    with pytest.raises(libfwi.FwiError) as err:
+        ctx.forward(m)
+    assert err.value.status == libfwi.FWI_ERR_CUDA
+    assert "column pass TMA staging: pipeline wait timed out (code 5)" in str(err.value)
+    assert 1.9 < waited < 4.0, waited
+    assert np.array_equal(to_np(ctx.apply("A", v, 1, m)), ref)
+    assert ctx.forward(m).info.n_not_converged == 0
+    ctx.close()
