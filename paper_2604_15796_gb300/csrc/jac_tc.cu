@@ -24,7 +24,11 @@
 // one warp issues the MMAs and
 // releases the stage with tcgen05.commit; two TMEM accumulators alternate so
 // that four more warps read one out while the MMAs fill the other.  Every
-// wait is bounded (tc.cuh).
+// wait is bounded (tc.cuh).  When one gives up, all run their loops to the end,
+// but a thread issues no copy and fills no stage unless its own wait for the
+// buffer succeeded, and the copies still in flight are waited for (bounded) at
+// the end; so a barrier is never armed again while its copy is pending, nothing
+// is written that MMAs may still read, and nothing lands after the CTA.
 //
 // What bounds a k-step (8 complex values of K, 128 x 128 complex outputs):
 // the six MMAs take 770 cycles at the TF32 rate, the operand traffic through
@@ -384,23 +388,26 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_contract_kernel(
     // the raw stage of step i - 1 is free after step i's barrier
 #pragma unroll
     for (int i = 0; i < (RN > 1 ? RN - 1 : 1); ++i) issue(i);
+    int failed_at = ni;  // first step whose raw tile this thread did not see arrive
     for (int i = 0; i < ni; ++i) {
       const int g = grp + GROUPS * i;
       const int slot = grp * RN + i % RN;
-      if (XTMA)
-        mbar_wait(smem_addr(&bar_raw[slot]), (i / RN) & 1, &abort_flag, p.err, kErrWaitFull);
+      if (XTMA &&
+          !mbar_wait(smem_addr(&bar_raw[slot]), (i / RN) & 1, &abort_flag, p.err, kErrWaitFull) &&
+          failed_at == ni)
+        failed_at = i;
       cp_async_wait<(RN > 1 ? RN - 2 : 0)>();
       bar_sync(1 + grp, 128);  // step i visible to the group; all done with step i - 1
-      if (RN > 1) issue(i + RN - 1);
+      if (RN > 1 && failed_at == ni) issue(i + RN - 1);
       const int cs = g % C_CONV;
-      mbar_wait(smem_addr(&bar_empty[cs]), ((g / C_CONV) & 1) ^ 1, &abort_flag, p.err,
-                kErrWaitEmpty);
+      const bool vacant = mbar_wait(smem_addr(&bar_empty[cs]), ((g / C_CONV) & 1) ^ 1,
+                                    &abort_flag, p.err, kErrWaitEmpty);
       const uint32_t rb = raw0 + (uint32_t)(slot * C_RAW_BYTES);
       const uint32_t ra = sbase + RW::AW + 64 * slot;
       const uint32_t cb = sbase + (uint32_t)(cs * C_CONV_BYTES);
       const uint32_t bhi = cb + 4 * PLANE, blo = bhi + bplane((uint32_t)nbr);
       // warps whose rows are all padding have nothing to convert
-      const bool work = r < ne || r < nbr;
+      const bool work = vacant && (r < ne || r < nbr);
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
         if (!work) break;
@@ -444,22 +451,17 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_contract_kernel(
         if (r < nbr) put_b(bhi, blo, half, r, nbr, qr, qi);
       }
       fence_proxy_async();
-      if (!(p.stall && g == 0)) mbar_arrive(smem_addr(&bar_full[cs]));
+      if (vacant && !(p.stall && g == 0)) mbar_arrive(smem_addr(&bar_full[cs]));
       if (RN == 1) {
         bar_sync(1 + grp, 128);  // the group's only raw stage is free
         issue(i + 1);
       }
     }
     cp_async_wait<0>();
-    if (XTMA && r == 0 && abort_flag) {
-      // copies issued before a wait gave up may still land in this CTA's
-      // shared memory: wait (bounded) for the last one of every raw stage
-      for (int k = 0; k < RN && k < ni; ++k) {
-        const int i = ni - 1 - ((ni - 1 - k) % RN);
+    if (XTMA && r == 0)  // the issued steps that were not seen to arrive
+      for (int i = failed_at; i < ni && i < failed_at + RN - 1; ++i)
         mbar_wait_drain(smem_addr(&bar_raw[grp * RN + i % RN]), (i / RN) & 1, p.err,
                         kErrWaitDrain);
-      }
-    }
   } else {
     int cs = 0, use = 0, ks = 0, sub = 0;  // stage, its use, k-step of the sub-chunk
     const KStep step((uint32_t)nbr);
@@ -525,6 +527,7 @@ struct JhArgs {
   long long N;
   int NE, n_freq, nbe, nks, npb, units;
   int conj_x;          // A = conj(X)^T (J^H) or X^T (adjoint sources)
+  int stall;           // test of the failure path: the MMA warp waits before its first unit
 };
 
 // FUSED: z_l[n] = s_l sum_e conj(X[e][n]) W[e][n] (J^H b); otherwise the
@@ -546,7 +549,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_jh_kernel(JhArgs p,
   __shared__ __align__(8) uint64_t bar_full[M_CONV], bar_empty[M_CONV], bar_done[2],
       bar_freed[2], bar_final, bar_raw[M_RAW];
   __shared__ uint32_t tmem_base;
-  __shared__ int abort_flag;
+  __shared__ int abort_flag, b_last[GROUPS];  // last step a group issued a B copy at
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int my_units = (blockIdx.x < p.units)
                            ? (p.units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1
@@ -647,7 +650,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_jh_kernel(JhArgs p,
     const int grp = tid / 128, r = tid % 128;
     // the group's k-steps g = grp + GROUPS i, i < ni, through its M_RN raw stages
     const int ni = (nchunks > grp) ? (nchunks - grp - 1) / GROUPS + 1 : 0;
-    auto issue = [&](int i) {
+    auto issue = [&](int i, bool go) {
       if (i < ni) {
         const int g = grp + GROUPS * i;
         int l, eb, pb;
@@ -657,7 +660,7 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_jh_kernel(JhArgs p,
         const uint32_t rb = raw0 + (uint32_t)(slot * M_RAW_BYTES);
         if (XTMA) {
           // rows j >= NE and pixels n >= N are outside the tensor: zero fill
-          if (r == 0) {
+          if (r == 0 && go) {
             const uint32_t bar = smem_addr(&bar_raw[slot]);
             mbar_arrive_expect_tx(bar, M_RAW_BYTES);
             tma_load_3d(rb, &xmap, 2 * pb * ROWS, ks * KS, l, bar);
@@ -679,22 +682,30 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_jh_kernel(JhArgs p,
       if (!XTMA) cp_async_commit();
     };
 #pragma unroll
-    for (int i = 0; i < M_RN - 1; ++i) issue(i);
+    for (int i = 0; i < M_RN - 1; ++i) issue(i, true);
+    // where this thread's waits first gave up: 2 i at the raw tile of step i (no
+    // further tile is issued), 2 i + 1 at its stage; step i and all later ones are
+    // skipped (every later wait gives up at once)
+    int stop = 2 * ni;
     for (int i = 0; i < ni; ++i) {
       const int g = grp + GROUPS * i;
       const int slot = grp * M_RN + i % M_RN;
-      if (XTMA)
-        mbar_wait(smem_addr(&bar_raw[slot]), (i / M_RN) & 1, &abort_flag, p.err, kErrWaitFull);
-      else
+      if (!XTMA)
         cp_async_wait<M_RN - 2>();
+      else if (!mbar_wait(smem_addr(&bar_raw[slot]), (i / M_RN) & 1, &abort_flag, p.err,
+                          kErrWaitFull))
+        stop = min(stop, 2 * i);
       bar_sync(1 + grp, 128);
-      issue(i + M_RN - 1);
+      issue(i + M_RN - 1, stop == 2 * ni);
       const int kunit = g / p.nks, ks = g % p.nks;
       int l, eb, pb;
       unit_of(kunit, l, eb, pb);
       const int cs = g % M_CONV;
-      mbar_wait(smem_addr(&bar_empty[cs]), ((g / M_CONV) & 1) ^ 1, &abort_flag, p.err,
-                kErrWaitEmpty);
+      if (!mbar_wait(smem_addr(&bar_empty[cs]), ((g / M_CONV) & 1) ^ 1, &abort_flag, p.err,
+                     kErrWaitEmpty)) {
+        stop = min(stop, 2 * i + 1);
+        continue;
+      }
       const uint32_t cb = sbase + (uint32_t)(cs * M_CONV_BYTES);
       if (r == 0) {
         const uint32_t fb = smem_addr(&bar_full[cs]);
@@ -720,16 +731,21 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_jh_kernel(JhArgs p,
       fence_proxy_async();
       mbar_arrive(smem_addr(&bar_full[cs]));
     }
+    // a stage with a B copy (of a step r = 0 did not skip) gets the arrivals of the
+    // threads that skipped it, so that its barrier completes with the copy (a
+    // barrier of the copy's own, which the MMA warp waited for as well, cost 7 %:
+    // 659 -> 708 us a launch at 384^2 pixels x 192 elements x 3 frequencies)
+    if (r == 0) b_last[grp] = stop / 2 - 1;
+    bar_sync(1 + grp, 128);
+    for (int i = stop / 2; i <= b_last[grp]; ++i)
+      mbar_arrive(smem_addr(&bar_full[(grp + GROUPS * i) % M_CONV]));
     if (!XTMA) {
       cp_async_wait<0>();
-    } else if (r == 0 && abort_flag) {
-      // copies issued before a wait gave up may still land in this CTA's
-      // shared memory: wait (bounded) for the last one of every raw stage
-      for (int k = 0; k < M_RN && k < ni; ++k) {
-        const int i = ni - 1 - ((ni - 1 - k) % M_RN);
+    } else if (r == 0) {  // the issued tiles that were not seen to arrive
+      const int k = (stop + 1) / 2;
+      for (int i = k; i < ni && i < k + M_RN - 1; ++i)
         mbar_wait_drain(smem_addr(&bar_raw[grp * M_RN + i % M_RN]), (i / M_RN) & 1, p.err,
                         kErrWaitDrain);
-      }
     }
   } else {
     int cs = 0, use = 0, ks = 0, kunit = 0;
@@ -740,6 +756,8 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_jh_kernel(JhArgs p,
         int l, eb, pb;
         unit_of(kunit, l, eb, pb);
         step = KStep((uint32_t)jh_rows(p.NE, eb));
+        if (p.stall && kunit == 0)  // for what completes after its last one
+          mbar_wait(smem_addr(&bar_final), 0, &abort_flag, p.err, kErrWaitDone);
         if (kunit >= 2) {
           // buffer b is free once unit kunit - 2 has been read out
           mbar_wait(smem_addr(&bar_freed[b]), ((kunit - 2) >> 1) & 1, &abort_flag, p.err,
@@ -769,7 +787,19 @@ __global__ void __launch_bounds__(C_THREADS, 1) tc_jh_kernel(JhArgs p,
   __syncthreads();
   if (warp == 0) {
     fence_after_sync();
-    if (lane == 0) mbar_wait_drain(smem_addr(&bar_final), 0, p.err, kErrWaitDrain);
+    if (lane == 0) {
+      mbar_wait_drain(smem_addr(&bar_final), 0, p.err, kErrWaitDrain);
+      if (abort_flag) {  // the last B copy into each stage
+        uint32_t armed[M_CONV] = {};
+        for (int grp = 0; grp < GROUPS; ++grp)
+          for (int i = b_last[grp]; i >= 0 && i > b_last[grp] - M_CONV; --i) {
+            const int g = grp + GROUPS * i;
+            armed[g % M_CONV] = max(armed[g % M_CONV], (uint32_t)(g / M_CONV + 1));
+          }
+        for (int cs = 0; cs < M_CONV; ++cs)
+          mbar_drain_armed(smem_addr(&bar_full[cs]), armed[cs], p.err, kErrWaitDrain);
+      }
+    }
     __syncwarp();
     tmem_dealloc(tmem, 512);
   }
@@ -971,7 +1001,8 @@ int tc_mix(fwi_ctx* c, const V* B, const float2* X, const float2* Xe, int conj_x
   const int units = c->n_freq * nbe * npb;
   const int grid = units < c->n_sm ? units : c->n_sm;
   JhArgs args{X, Xe, (const float*)c->tc_bops, c->red, out, c->tc_err, c->N,
-              c->n_elem, c->n_freq, nbe, nks, npb, units, conj_x};
+              c->n_elem, c->n_freq, nbe, nks, npb, units, conj_x, c->tc_stall};
+  c->tc_stall = 0;  // one launch
   // the mixed operand [n_freq][NE][N] as a 3-D tensor of floats, box 8 rows
   // (one k-step of j) x 128 pixels
   CUtensorMap xmap;

@@ -154,8 +154,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 
 // Wait for the phase of parity `parity` to complete.  Gives up after
 // kWaitLimitNs: sets *abort (shared) and the error word, returns false.
-// Once *abort is set every later wait returns at once, so all threads run
-// their loops to the end and the block exits.
+// Once *abort is set every later wait returns false at once, so all threads
+// run their loops to the end and the block exits.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort,
                                           int* err, int code) {
   if (*abort) return false;

@@ -39,3 +39,40 @@ def test_stalled_spectrum_copy_is_waited_for(pairs, n_rhs):
     assert np.array_equal(to_np(ctx.apply("A", v, 1, m)), ref)
     assert ctx.forward(m).info.n_not_converged == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("tma", [True, False])
+@pytest.mark.parametrize("n_elem", [61, 129])
+def test_stalled_contraction_leaves_no_copy_behind(n_elem, tma):
+    """The contraction (54 and 216 k-steps per CTA) and J^H (32 and 119, B blocks by
+    bulk copies) stall at their first stage with their rings of raw tiles full: the
+    producers stop at their next barrier instead of arming tiles whose copies are
+    pending, the waits run out once (1 s), and the next calls give the same bits."""
+    import torch
+    from paper_2604_15796_gb300 import build, libfwi
+    build.build()
+    w = phantoms.scaled((256, 256), 0.1e-3, n_elem, 25e-3 / n_elem, np.array([1.0e6]), 11,
+                        inclusions=[1520.0, 1580.0])
+    ctx = libfwi.Context(w.shape, w.h, w.c0, w.elem, w.freqs)
+    ctx.set_jac_tma(tma)
+    m = to_gpu(contrast(w), torch.complex128)
+    ctx.forward(m)
+    a = to_gpu(phantoms.complex_normal(w.shape, 5), torch.complex128)
+    b = to_gpu(phantoms.complex_normal((1, n_elem, n_elem), 6), torch.complex128)
+    grad = torch.empty(w.shape, dtype=torch.complex128, device="cuda")
+    zero = torch.zeros((1, n_elem, n_elem), dtype=torch.complex64, device="cuda")
+    calls = {"J a": lambda: to_np(ctx.jac_forward(a)), "J^H b": lambda: to_np(ctx.jac_adjoint(b))}
+    ref = {k: f() for k, f in calls.items()}
+    for k, f in calls.items():
+        ctx.debug_stall_once()
+        t0 = time.perf_counter()
+        f()
+        waited = time.perf_counter() - t0
+        with pytest.raises(libfwi.FwiError) as err:
+            ctx.forward(m)
+        assert "tensor-core contraction: pipeline wait timed out" in str(err.value)
+        assert 0.9 < waited < 1.8, (k, waited)
+        ctx.gradient(m, zero, grad)
+        for k2, f2 in calls.items():
+            assert np.array_equal(f2(), ref[k2]), (k, k2)
+    ctx.close()
