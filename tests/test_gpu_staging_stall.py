@@ -46,8 +46,9 @@ def test_stalled_spectrum_copy_is_waited_for(pairs, n_rhs):
 def test_stalled_contraction_leaves_no_copy_behind(n_elem, tma):
     """The contraction (54 and 216 k-steps per CTA) and J^H (32 and 119, B blocks by
     bulk copies) stall at their first stage with their rings of raw tiles full: the
-    producers stop at their next barrier instead of arming tiles whose copies are
-    pending, the waits run out once (1 s), and the next calls give the same bits."""
+    waits run out once (1 s), no tile is issued again while its copy is pending,
+    every copy in flight is seen to land (a second limit would double the time), and
+    the next calls give the same bits."""
     import torch
     from paper_2604_15796_gb300 import build, libfwi
     build.build()
