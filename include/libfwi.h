@@ -478,8 +478,9 @@ typedef struct fwi_tuning {
                            stages its kernel-spectrum tiles with TMA (half
                            the column's rows, the spectrum being even; one
                            column per thread: where they fit); 0: the
-                           spectrum is read from global memory.  Results
-                           agree to FP32 rounding. */
+                           spectrum is read from global memory, one column
+                           per thread unless the transform length is 16, 64,
+                           256 or 512.  Results agree to FP32 rounding. */
   int jac_tma;          /* 1 (default): the tensor-core pixel contractions
                            receive their raw FP32 operand tiles by TMA
                            tensor copies issued by one producer thread;
@@ -496,12 +497,13 @@ typedef struct fwi_tuning {
                            samples there; 0: loads from global memory (with
                            row_l2_prefetch).  Results agree to FP32
                            rounding. */
-  int col_pairs;        /* 1 (default): the FP32 convolution pass, where its
-                           kernel spectrum is staged (col_tma and
-                           col_spectrum_stage), computes two columns per
-                           thread with packed f32x2 arithmetic on column
-                           pairs; 0: one column per thread.  Results agree
-                           to FP32 rounding. */
+  int col_pairs;        /* 1 (default): the FP32 convolution pass, with
+                           col_tma, computes two columns per thread with
+                           packed f32x2 arithmetic on column pairs (with
+                           col_spectrum_stage at every transform length,
+                           without it at 16, 64, 256 and 512 points); 0: one
+                           column per thread.  Results agree to FP32
+                           rounding. */
 } fwi_tuning;
 FWI_API fwi_status fwi_get_tuning(const fwi_ctx* ctx, fwi_tuning* out);
 FWI_API fwi_status fwi_set_tuning(fwi_ctx* ctx, const fwi_tuning* in);

@@ -1,4 +1,5 @@
-// Convolution pass with two columns per thread (FP32, every transform length).
+// Convolution pass with two columns per thread (FP32, every transform length;
+// with its spectrum read from L2 instead of staged, the lengths of pair_l2()).
 //
 // The transforms are the four-step FFT of fft_core.cuh (forward FFT along
 // the column with the zero-padded half pruned, product with the kernel
@@ -285,8 +286,8 @@ template <> struct PairPlanFor<1024> { using type = Plan<1024, 32, 32, 32>; };
 // Shared memory (bytes from the 128-byte aligned base): exchange, R2 rows of
 // R1 (+ 1 for tiles under 8 pairs, whose rows would otherwise start in the same
 // banks) x NP pairs of 16 bytes | input staging rows_in x TC (unless it lies in
-// the exchange) | kernel-spectrum tile, rows 0..L/2 in GBOX boxes of at most 256
-// rows | twiddle table L | two mbarriers and the abort flag.
+// the exchange) | kernel-spectrum tile (where staged), rows 0..L/2 in GBOX boxes
+// of at most 256 rows | twiddle table L | two mbarriers and the abort flag.
 // ALIAS: the input staging lies inside the exchange buffer (free until every
 // thread holds its samples) where a separate one would leave one CTA per SM;
 // the next item's copy then starts when the inverse transforms have read the
@@ -304,9 +305,9 @@ template <class P, int TC> struct ColPairSmem {
   static_assert(P::R2 * R1P * ROW % 128 == 0 && P::L / 2 * ROW % 128 == 0 &&
                 (GBOX == 1 || G_BOX_ROWS * ROW % 128 == 0) && G_ROWS <= P::L &&
                 G_BOX_ROWS <= 256, "TMA destinations and boxes");
-  static constexpr size_t bytes(int rows_in) {
+  static constexpr size_t bytes(int rows_in, bool gs) {
     return ((size_t)P::R2 * R1P * TC + (ALIAS ? 0 : (size_t)rows_in * TC) +
-            (size_t)G_ROWS * TC + (size_t)P::L) * sizeof(float2) + 32 + 128;
+            (gs ? (size_t)G_ROWS * TC : 0) + (size_t)P::L) * sizeof(float2) + 32 + 128;
   }
 };
 
@@ -326,7 +327,14 @@ __host__ __device__ constexpr unsigned pair_group(unsigned ntile) {
 template <class P> constexpr int pair_blocks(int threads) {
   return P::E > 24 ? 2 * (128 / threads > 1 ? 128 / threads : 1) : blocks_for_regs(threads, 168);
 }
-template <class P, int TC>
+// GS: the spectrum is staged as above; otherwise (col_spectrum_stage = 0) every
+// thread reads its column pairs from global memory (L2), at the lengths where
+// that was measured against one column per thread, a launch: 16 points (8 x 512
+// pixels, 1,024 right-hand sides) 49.2 -> 43.6 us, 64 (32 x 256, 1,024) 95.8 ->
+// 79.1, 256 (128 x 256, 1,024) 464 -> 351 and (128 x 160 x 160, 16) 1,343 ->
+// 1,182, 512 (256 x 256, 512) 600 -> 422; staged: 42.6, 77, 327, 1,003 and 403.
+template <int L> constexpr bool pair_l2() { return L == 16 || L == 64 || L == 256 || L == 512; }
+template <class P, int TC, bool GS>
 __global__ void __launch_bounds__(TC / 2 * P::TL, pair_blocks<P>(TC / 2 * P::TL))
 col_pair_kernel(const ColArgs<float> a, const __grid_constant__ CUtensorMap map,
                 const __grid_constant__ CUtensorMap gmap, int rows_in, int nbox) {
@@ -342,7 +350,7 @@ col_pair_kernel(const ColArgs<float> a, const __grid_constant__ CUtensorMap map,
   float2* ex_end = reinterpret_cast<float2*>(ex + R2 * R1P * NP);
   float2* stg = ALIAS ? reinterpret_cast<float2*>(ex) : ex_end;    // input staging
   float2* gst = ex_end + (ALIAS ? 0 : rows_in * TC);               // spectrum staging
-  float2* tws = gst + SM::G_ROWS * TC;                             // twiddles
+  float2* tws = gst + (GS ? SM::G_ROWS * TC : 0);                  // twiddles
   uint64_t* bar = reinterpret_cast<uint64_t*>(tws + P::L);         // [0] input, [1] spectrum
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bar + 2);
   const uint32_t bar_in = tc::smem_addr(bar), bar_g = tc::smem_addr(bar + 1);
@@ -410,11 +418,11 @@ col_pair_kernel(const ColArgs<float> a, const __grid_constant__ CUtensorMap map,
   Item it = first < last ? item_of(first) : Item{0, 0, 0, 0}, nx = it;
   if (threadIdx.x == 0 && first < last) {
     issue_input(it);
-    issue_spectrum(it);
+    if (GS) issue_spectrum(it);
   }
   uint32_t par_in = 0, par_g = 0;
   // new_g: the item has another spectrum tile than the one before it
-  bool failed = false, bad = false, new_g = true;
+  bool failed = false, bad = false, new_g = GS;
   for (unsigned item = first; item < last; ++item, it = nx) {
     const bool more = item + 1 < last;
     if (more) nx = item_of(item + 1);
@@ -469,7 +477,11 @@ col_pair_kernel(const ColArgs<float> a, const __grid_constant__ CUtensorMap map,
     }
     __syncthreads();
     // phase B: R2-point DFTs over n2, v[k2] = X[k1 + R1 k2]; product with the
-    // kernel spectrum (rows folded onto 0..L/2)
+    // kernel spectrum (rows folded onto 0..L/2): the staged tile, or columns
+    // (j, j + 1) of the item's frequency
+    const float4* __restrict__ gg = nullptr;
+    if constexpr (!GS)
+      gg = reinterpret_cast<const float4*>(a.ghat + (long long)it.l * a.ghat_freq_stride + j);
 #pragma unroll
     for (int i = 0; i < C3; ++i) {
       const int k1 = t + i * TL;
@@ -481,14 +493,16 @@ col_pair_kernel(const ColArgs<float> a, const __grid_constant__ CUtensorMap map,
 #pragma unroll
       for (int k2 = 0; k2 < R2; ++k2) {
         const int row = spectrum_row<P>(k1, k2, k2);
-        const float4 g = gst4[row * NP + cp];
+        float4 g;
+        if constexpr (GS) g = gst4[row * NP + cp];
+        else g = __ldg(gg + (long long)row * (a.ncols / 2));
         u[k2] = pmul(u[k2], pk(g.x, g.z), pk(g.y, g.w));
       }
     }
     // The exchange slots (n2, k1) of a k1 belong to its thread in phases B and
     // C alike, so no barrier separates them; one before the next item's spectrum
     // tile replaces this one.
-    new_g = more && (nx.tile != it.tile || nx.l != it.l);
+    new_g = GS && more && (nx.tile != it.tile || nx.l != it.l);
     if (new_g) {
       tc::fence_proxy_async();
       __syncthreads();

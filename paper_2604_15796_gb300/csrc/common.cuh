@@ -92,7 +92,7 @@ template <typename T> struct ColArgs {
   int freq_fixed;           // >= 0: every RHS uses this frequency
   int tma;                  // FP32, zero-padded input: stage tiles with TMA
   int gstage;               // with tma: also stage the kernel-spectrum tiles
-  int pairs;                // with gstage: two columns per thread where the plan allows
+  int pairs;                // with tma: two columns per thread where there is a kernel for it
   int stall;                // test of the failure path: spectrum copies announce too many bytes
   int* err;                 // error word of bounded waits (or NULL)
 };

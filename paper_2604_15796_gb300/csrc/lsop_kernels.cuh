@@ -1414,8 +1414,7 @@ bool col_tensor_map(const ColArgs<float>& a, CUtensorMap* map, int* rows_in, int
   return true;
 }
 
-// The two-column convolution stores 16-byte column pairs, and takes its
-// spectrum from a staged tile.
+// The two-column convolution stores 16-byte column pairs.
 template <typename T> bool col_pair_ok(const ColArgs<T>& a) {
   return a.mode == C_CONV && a.pairs && a.ghat && ((uintptr_t)a.out & 15) == 0 &&
          a.out_rhs_stride % 2 == 0 && a.line_stride % 2 == 0 &&
@@ -1435,8 +1434,8 @@ cudaError_t launch_col(const ColArgs<T>& a, cudaStream_t s) {
         using PP = typename PairPlanFor<L>::type;
         using PSM = ColPairSmem<PP, tc>;
         if (col_pair_ok(a) && col_spectrum_map<L, tc>(a, PSM::G_BOX_ROWS, &gmap)) {
-          auto k = col_pair_kernel<PP, tc>;
-          const size_t smem = PSM::bytes(rows_in);
+          auto k = col_pair_kernel<PP, tc, true>;
+          const size_t smem = PSM::bytes(rows_in, true);
           GridCache& gc = gcache<L, T, 6, VAR>();
           cudaError_t e = grid_for(k, tc / 2 * PP::TL, smem, gc);
           if (e != cudaSuccess) return e;
@@ -1465,6 +1464,19 @@ cudaError_t launch_col(const ColArgs<T>& a, cudaStream_t s) {
       {
         cudaError_t e = grid_for(kp, tc * P::TL, col_smem_v<L, T, VAR>(), gcp);
         if (e != cudaSuccess) return e;
+      }
+      if constexpr (pair_l2<L>() && tc % 2 == 0) {
+        // the spectrum from global memory (16-byte column pairs)
+        if (col_pair_ok(a) && al16(a.ghat) && a.ncols % 2 == 0 && a.ghat_freq_stride % 2 == 0) {
+          using PP = typename PairPlanFor<L>::type;
+          auto k = col_pair_kernel<PP, tc, false>;
+          const size_t smem = ColPairSmem<PP, tc>::bytes(rows_in, false);
+          GridCache& gc = gcache<L, T, 7, VAR>();
+          cudaError_t e = grid_for(k, tc / 2 * PP::TL, smem, gc);
+          if (e != cudaSuccess) return e;
+          k<<<gc.blocks.load(), tc / 2 * PP::TL, smem, s>>>(a, map, gmap, rows_in, nbox);
+          return cudaGetLastError();
+        }
       }
       auto k = col_tma_kernel<P, tc, false>;
       const size_t smem = SM::bytes(rows_in, false);
