@@ -467,8 +467,10 @@ fwi_status fwi_adjoint(fwi_ctx* ctx, const void* m, const void* src, void* lambd
   if (st != FWI_OK && st != FWI_ERR_NOT_CONVERGED) return st;
   fwi_status st2 = copy_field(ctx, lambda, ctx->lam, (long long)ctx->n_rhs * ctx->N, 1);
   if (st2 == FWI_OK) {
+    tc_err_fetch(ctx);  // a staged pass of the solve may have given up
     cudaError_t e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "fwi_adjoint");
+    st2 = tc_err_check(ctx);
   }
   return st2 != FWI_OK ? st2 : st;
 }

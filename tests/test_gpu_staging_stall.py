@@ -77,3 +77,27 @@ def test_stalled_contraction_leaves_no_copy_behind(n_elem, tma):
         for k2, f2 in calls.items():
             assert np.array_equal(f2(), ref[k2]), (k, k2)
     ctx.close()
+
+
+def test_adjoint_reports_a_wait_that_gave_up():
+    """The error word is reported by the next call that synchronises, the adjoint
+    solve among them."""
+    import torch
+    from paper_2604_15796_gb300 import build, libfwi
+    build.build()
+    w = small_workload((32, 32), n_elem=6)
+    ctx = libfwi.Context(w.shape, w.h, w.c0, w.elem, w.freqs)
+    m = to_gpu(contrast(w), torch.complex128)
+    v = to_gpu(phantoms.complex_normal((w.n_freq, 6) + tuple(w.shape), 3), torch.complex64)
+    ref = ctx.empty_fields()
+    ctx.adjoint(m, v, ref)
+    ctx.debug_stall_once()
+    ctx.apply("K", v[0], 0)
+    lam = ctx.empty_fields()
+    with pytest.raises(libfwi.FwiError) as err:
+        ctx.adjoint(m, v, lam)
+    assert err.value.status == libfwi.FWI_ERR_CUDA
+    assert "column pass TMA staging: pipeline wait timed out" in str(err.value)
+    ctx.adjoint(m, v, lam)
+    ctx.close()
+    assert torch.equal(lam, ref)
