@@ -50,12 +50,11 @@ __device__ inline void tile_of(int ty, int nbe, int sym, int& eb, int& jb) {
 }
 
 // FP32 fields on CUDA cores.
-template <typename T>
 __global__ void __launch_bounds__(256)
-contract_kernel(const cplx<T>* __restrict__ X, const cplx<T>* __restrict__ a,
-                const cplx<T>* __restrict__ Q, cplx<T>* __restrict__ part, int NE,
+contract_kernel(const float2* __restrict__ X, const float2* __restrict__ a,
+                const float2* __restrict__ Q, float2* __restrict__ part, int NE,
                 long long N, int n_freq, long long chunk, int sym) {
-  using V = cplx<T>;
+  using V = float2;
   __shared__ V Xs[KC][TB + 1];
   __shared__ V Qs[KC][TB + 1];
   const int s = blockIdx.x;
@@ -74,7 +73,7 @@ contract_kernel(const cplx<T>* __restrict__ X, const cplx<T>* __restrict__ a,
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = mk<T>(T(0), T(0));
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
   for (long long n0 = n_begin; n0 < n_end; n0 += KC) {
 #pragma unroll
     for (int q = 0; q < (TB * KC) / 256; ++q) {
@@ -82,7 +81,7 @@ contract_kernel(const cplx<T>* __restrict__ X, const cplx<T>* __restrict__ a,
       const int r = idx / KC, cc = idx % KC;
       const long long n = n0 + cc;
       const int e = eb * TB + r, j = jb * TB + r;
-      V xv = mk<T>(T(0), T(0)), qv = mk<T>(T(0), T(0));
+      V xv = make_float2(0.f, 0.f), qv = make_float2(0.f, 0.f);
       if (n < n_end) {
         if (e < NE) {
           xv = Xl[(long long)e * N + n];
@@ -280,12 +279,13 @@ cudaError_t contract_reduce(fwi_ctx* c, double2* Y, int split, long long per, in
   return cudaGetLastError();
 }
 
-template <typename T, bool FUSED>
+// FP32 fields on CUDA cores.
+template <bool FUSED>
 __global__ void __launch_bounds__(256)
-mix_kernel(const cplx<T>* __restrict__ B, const cplx<T>* __restrict__ Q, int conjQ,
-           const cplx<T>* __restrict__ X, cplx<T>* __restrict__ out,
+mix_kernel(const float2* __restrict__ B, const float2* __restrict__ Q, int conjQ,
+           const float2* __restrict__ X, float2* __restrict__ out,
            const double* __restrict__ scale, int NE, long long N) {
-  using V = cplx<T>;
+  using V = float2;
   __shared__ V Bs[KC][TB + 1];
   __shared__ V Qs[KC][TB + 1];
   __shared__ V red[16][TB + 1];
@@ -300,7 +300,7 @@ mix_kernel(const cplx<T>* __restrict__ B, const cplx<T>* __restrict__ Q, int con
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = mk<T>(T(0), T(0));
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
   for (int j0 = 0; j0 < NE; j0 += KC) {
 #pragma unroll
     for (int q = 0; q < (TB * KC) / 256; ++q) {
@@ -309,14 +309,14 @@ mix_kernel(const cplx<T>* __restrict__ B, const cplx<T>* __restrict__ Q, int con
       {
         const int r = idx / KC, cc = idx % KC;
         const int e = eb * TB + r, j = j0 + cc;
-        Bs[cc][r] = (e < NE && j < NE) ? Bl[(long long)e * NE + j] : mk<T>(T(0), T(0));
+        Bs[cc][r] = (e < NE && j < NE) ? Bl[(long long)e * NE + j] : make_float2(0.f, 0.f);
       }
       // Q tile: row j (KC of them), TB consecutive n
       {
         const int kk = idx / TB, nn = idx % TB;
         const int j = j0 + kk;
         const long long n = n0 + nn;
-        V v = mk<T>(T(0), T(0));
+        V v = make_float2(0.f, 0.f);
         if (j < NE && n < N) {
           v = Ql[(long long)j * N + n];
           if (conjQ) v.y = -v.y;
@@ -342,7 +342,7 @@ mix_kernel(const cplx<T>* __restrict__ B, const cplx<T>* __restrict__ Q, int con
     }
     __syncthreads();
   }
-  const T f = (T)scale[l];
+  const float f = (float)scale[l];
   if (!FUSED) {
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -351,7 +351,7 @@ mix_kernel(const cplx<T>* __restrict__ B, const cplx<T>* __restrict__ Q, int con
         const int e = eb * TB + te + 16 * i;
         const long long n = n0 + tn + 16 * j;
         if (e < NE && n < N)
-          out[((long long)l * NE + e) * N + n] = mk<T>(acc[i][j].x * f, acc[i][j].y * f);
+          out[((long long)l * NE + e) * N + n] = make_float2(acc[i][j].x * f, acc[i][j].y * f);
       }
     return;
   }
@@ -360,7 +360,7 @@ mix_kernel(const cplx<T>* __restrict__ B, const cplx<T>* __restrict__ Q, int con
   V zs[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    zs[j] = mk<T>(T(0), T(0));
+    zs[j] = make_float2(0.f, 0.f);
     const long long n = n0 + tn + 16 * j;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -374,11 +374,11 @@ mix_kernel(const cplx<T>* __restrict__ B, const cplx<T>* __restrict__ Q, int con
   }
   __syncthreads();
   if (tid < TB) {
-    V s = mk<T>(T(0), T(0));
+    V s = make_float2(0.f, 0.f);
 #pragma unroll
     for (int r = 0; r < 16; ++r) s = cadd(s, red[r][tid]);
     const long long n = n0 + tid;
-    if (n < N) out[((long long)l * nbe + eb) * N + n] = mk<T>(s.x * f, s.y * f);
+    if (n < N) out[((long long)l * nbe + eb) * N + n] = make_float2(s.x * f, s.y * f);
   }
 }
 
@@ -523,8 +523,8 @@ template <typename T> struct Jac {
         contract_f64_kernel<<<dim3(tiles, split, c->n_freq), TD * TD, 0, c->stream>>>(
             X, a, Q, (double2*)c->jsplit, c->n_elem, c->N, c->n_freq, chunk, sym);
       else
-        contract_kernel<T><<<grid, 256, 0, c->stream>>>(X, a, Q, (cplx<T>*)c->jsplit, c->n_elem,
-                                                        c->N, c->n_freq, chunk, sym);
+        contract_kernel<<<grid, 256, 0, c->stream>>>(X, a, Q, (float2*)c->jsplit, c->n_elem,
+                                                     c->N, c->n_freq, chunk, sym);
     }
     FWI_CUDA(c, cudaGetLastError());
     Prof p(c, KC_MISC);
@@ -722,8 +722,8 @@ template <typename T> static fwi_status adjoint_sources_t(fwi_ctx* c, void* out)
         (const double2*)c->dF, (const double2*)c->p0, 0, nullptr, (double2*)out, c->red,
         c->n_elem, c->N);
   } else {
-    mix_kernel<T, false><<<grid, 256, 0, c->stream>>>(
-        (const cplx<T>*)c->dF, (const cplx<T>*)c->p0, 0, nullptr, (cplx<T>*)out, c->red,
+    mix_kernel<false><<<grid, 256, 0, c->stream>>>(
+        (const float2*)c->dF, (const float2*)c->p0, 0, nullptr, (float2*)out, c->red,
         c->n_elem, c->N);
   }
   FWI_CUDA(c, cudaGetLastError());
@@ -828,9 +828,9 @@ template <typename T> static fwi_status jac_adjoint_t(fwi_ctx* c, const double2*
           (const double2*)c->dF, (const double2*)receiver_fields(c), 1,
           (const double2*)c->fields, (double2*)c->zpart, c->red, c->n_elem, c->N);
     } else {
-      mix_kernel<T, true><<<grid, 256, 0, c->stream>>>(
-          (const cplx<T>*)c->dF, (const cplx<T>*)receiver_fields(c), 1,
-          (const cplx<T>*)c->fields, (cplx<T>*)c->zpart, c->red, c->n_elem, c->N);
+      mix_kernel<true><<<grid, 256, 0, c->stream>>>(
+          (const float2*)c->dF, (const float2*)receiver_fields(c), 1,
+          (const float2*)c->fields, (float2*)c->zpart, c->red, c->n_elem, c->N);
     }
   }
   FWI_CUDA(c, cudaGetLastError());
@@ -987,9 +987,8 @@ extern "C" fwi_status fwi_contract_pixels_noalloc(const void* X, const void* a, 
   FreqScales sc{};
   for (int l = 0; l < n_freq; ++l) sc.s[l] = scale[l];
   dim3 grid((unsigned)split, nbe * nbe, n_freq);
-  contract_kernel<float><<<grid, 256, 0, s>>>((const float2*)X, (const float2*)a,
-                                              (const float2*)Q, part, n_elem, N, n_freq, chunk,
-                                              0);
+  contract_kernel<<<grid, 256, 0, s>>>((const float2*)X, (const float2*)a, (const float2*)Q,
+                                       part, n_elem, N, n_freq, chunk, 0);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "fwi_contract_pixels_noalloc launch");
   contract_reduce_static_kernel<<<blocks_for(per, 256, sms * 8), 256, 0, s>>>(

@@ -899,12 +899,6 @@ cudaError_t set_attrs() {
   return g_attr_err;
 }
 
-// Shared launcher of the two mixes; B is [n_freq][NE][NE] (double2 for
-// J^H, float2 for the adjoint sources).
-template <bool FUSED, typename V>
-int tc_mix(fwi_ctx* c, const V* B, const float2* X, int conj_x, float2* out, int kclass,
-           double bytes, double flops);
-
 }  // namespace
 
 bool tc_usable(const fwi_ctx* c) {
@@ -976,6 +970,8 @@ int tc_contract_partials(fwi_ctx* c, const float2* X, const float2* a, const flo
 
 namespace {
 
+// Shared launcher of the two mixes; B is [n_freq][NE][NE] (double2 for
+// J^H, float2 for the adjoint sources).
 template <bool FUSED, typename V>
 int tc_mix(fwi_ctx* c, const V* B, const float2* X, const float2* Xe, int conj_x, float2* out,
            int kclass, double bytes, double flops) {
