@@ -227,7 +227,8 @@ mix_f64_kernel(const double2* __restrict__ B, const double2* __restrict__ Q, int
 // sym, entries below the computed tiles (eb > jb) are read transposed.
 // LANES (a power of two up to 32) neighbouring threads share one output, each
 // adding every LANES-th partial: 8 where there are few outputs and many splits,
-// whose loads would otherwise form one serial chain per output.
+// whose loads would otherwise form one serial chain per output (see
+// contract_reduce for where the line lies).
 template <typename T, int LANES>
 __global__ void contract_reduce_kernel(double2* Y, const cplx<T>* part, int split,
                                        long long per_split, int NE2, const double* scale,
@@ -266,6 +267,11 @@ __global__ void contract_reduce_kernel(double2* Y, const cplx<T>* part, int spli
 
 // Reduction of the split partials; sym_tile: the tile edge when only tiles on
 // and above the diagonal were computed, else 0.
+// 8 lanes an output below 16,384 outputs (from 16 partials on): one J a's kernels
+// beside the contraction with 1 and with 8 lanes, us: 256 outputs x 152 partials
+// 55, 18; 4,096 x 152: 57, 19; 8,192 x 76: 35, 20; 16,384 x 38: 25, 20; 16,384 x
+// 152: 58, 37.  Above, the threads of one lane each fill the chip, and 8 lanes read
+// the partials in smaller pieces: 32,768 x 76: 35, 39; 65,536 x 38: 35, 41.
 template <typename T>
 cudaError_t contract_reduce(fwi_ctx* c, double2* Y, int split, long long per, int sym_tile) {
   const int ne = c->n_elem;

@@ -445,10 +445,13 @@ __host__ __device__ inline int rf_stage_count(int mode, int use_m) {
 }
 
 // The forward row pass is latency-bound on its loads: the minimum-blocks
-// bound keeps it at <= 72 registers (no spills) so that more warps are
-// resident (10-14 % faster than the unconstrained 80-95 registers).  Lines
-// that do not tile a warp (TL = 20, 24: the 3-D x lines) hold more samples
-// per thread and get 88 (72 spilled 168 bytes per thread).
+// bound keeps it at <= 72 registers so that more warps are resident (10-14 %
+// faster than the unconstrained 80-95 registers).  Lines that do not tile a
+// warp (TL = 20, 24: the 3-D x lines) hold more samples per thread and get 88
+// (72 spilled 168 bytes per thread at 320 points).  Some plans spill at these
+// bounds (-Xptxas -v, bytes of spill stores, plain / staged): 128 points 40 / 32,
+// 256 0 / 8, 320 28 / 24, 384 224 / 48, 512 12 / 12, 640 68 / 28, 768 332 / 28,
+// 1024 48-124 / 8-180 by lines per CTA.
 template <class P, typename T, int LPC, bool STG = false>
 __global__ void __launch_bounds__(LPC * P::TL,
                                   blocks_for_regs(LPC * P::TL,
