@@ -19,10 +19,11 @@
 // and stage the next item's input tile by TMA while the current item transforms;
 // bounded mbarrier waits with the error codes of col_tma_kernel.
 //
-// What bounds it: FP32 issue and shared-memory traffic about equally (1024
-// points, 16 columns on one SM: 8,400 cycles of packed FP32 and 7,500 of
-// shared-memory accesses against 16,600 taken), with few warps to overlap the
-// two.  Cycles per 16 columns on one SM before (one column per thread, or lane
+// What bounds it: FP32 and shared-memory traffic about equally (counters of one
+// launch, 64 right-hand sides of 512^2, 1024 points: per 16 columns on one SM 8,200
+// cycles of the FMA pipe and 7,500 of the shared-memory data pipe against 16,600
+// taken), with few warps (7.5 a SM, 0.54 eligible a cycle) to overlap the two.
+// Cycles per 16 columns on one SM before (one column per thread, or lane
 // pairs sharing the 32-point DFTs of 512, and a spectrum tile copied or read
 // for every item) and now: 128: 2,370 -> 1,930; 192: 3,930 -> 2,980 (96^3:
 // 3,600 -> 2,560); 256: 3,430 -> 3,210; 320: 6,050 -> 5,210; 384: 8,500 ->
